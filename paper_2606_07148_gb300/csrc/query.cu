@@ -9,12 +9,19 @@
 
 namespace {
 
-__global__ void k_count_ones(const uint8_t *a, int64_t n, unsigned long long *out) {
+// Members in a mask of 0/1 bytes (a is 16-byte aligned).
+__global__ void __launch_bounds__(256) k_count_ones(const uint8_t *a, int64_t n, unsigned long long *out) {
     unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        c += a[i] != 0;
-    c = (unsigned long long)abc::warp_sum64((long long)c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    const uint4 *a4 = reinterpret_cast<const uint4 *>(a);
+    for (int64_t i = t0; i < n / 16; i += nt) {
+        const uint4 q = __ldg(&a4[i]);
+        c += (unsigned long long)(__popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w));
+    }
+    for (int64_t i = n / 16 * 16 + t0; i < n; i += nt) c += a[i] != 0;
+    const unsigned long long v[1] = {c};
+    unsigned long long *const d[1] = {out};
+    abc::block_add<1>(v, d);
 }
 
 // Membership in internal order from the caller-order masks.
@@ -32,13 +39,18 @@ unsigned grid_of(const abcore_ctx *ctx, int64_t n) {
 
 }  // namespace
 
+// Enqueue the (alpha, beta)-core's masks into the peel's staging buffer (peel_finish reports how it went).
+static int stage_core(abcore_ctx *ctx, int32_t alpha, int32_t beta) {
+    ABC_TRY(peel_finish(ctx));
+    ABC_TRY(peel_prepare(ctx));
+    uint8_t *su = ctx->w.stage, *sv = ctx->w.stage + ctx->g.nU;
+    return peel_compute(ctx, alpha, beta, su, sv, false, prefer_pruned(ctx, alpha, beta));
+}
+
 // Members of the (alpha, beta)-core, with the masks left in the peel's staging buffer.
 int core_size(abcore_ctx *ctx, int32_t alpha, int32_t beta, int64_t *size) {
     const Graph &g = ctx->g;
-    ABC_TRY(peel_finish(ctx));
-    ABC_TRY(peel_prepare(ctx));
-    uint8_t *su = ctx->w.stage, *sv = ctx->w.stage + g.nU;
-    ABC_TRY(peel_compute(ctx, alpha, beta, su, sv, false, prefer_pruned(ctx, alpha, beta)));
+    ABC_TRY(stage_core(ctx, alpha, beta));
     unsigned long long *cnt = nullptr;
     ABC_TRY(ctx->alloc(&cnt, 1, "core size"));
     unsigned long long h = 0;
@@ -75,15 +87,15 @@ int alpha_offset(abcore_ctx *ctx, int32_t alpha, int32_t *beta_out) {
 int community(abcore_ctx *ctx, int32_t q_internal, int32_t alpha, int32_t beta, uint8_t *d_mask_u, uint8_t *d_mask_v,
               int64_t *size) {
     const Graph &g = ctx->g;
-    int64_t sz = 0;
-    ABC_TRY(core_size(ctx, alpha, beta, &sz));
+    ABC_TRY(stage_core(ctx, alpha, beta));
     uint8_t *alive = nullptr;
     ABC_TRY(ctx->alloc(&alive, (size_t)std::max<int64_t>(g.n(), 1), "community membership"));
     if (g.n() > 0)
         k_alive_internal<<<grid_of(ctx, g.n()), 256, 0, ctx->stream>>>(g.new2old, g.nU, g.n(), ctx->w.stage,
                                                                        ctx->w.stage + g.nU, alive);
     ctx->stats.launches++;
-    int rc = community_compute(ctx, alive, q_internal, d_mask_u, d_mask_v, size);
+    const int rc = community_compute(ctx, alive, q_internal, d_mask_u, d_mask_v, size);  // (waits for the stream)
     ctx->release(alive);
-    return rc;
+    const int prc = peel_finish(ctx);  // a failed peel leaves masks that mean nothing
+    return prc ? prc : rc;
 }
