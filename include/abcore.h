@@ -19,6 +19,9 @@
  *    ready, except abcore_compute / abcore_compute_batch with ABCORE_PTR_DEVICE | ABCORE_ASYNC,
  *    which return once the work is enqueued; abcore_sync then waits and reports its status.
  *  - A context is not thread-safe: use one context per host thread.
+ *  - A context keeps device memory it no longer needs for its next call, up to a 64th of the
+ *    device's memory, until it is destroyed or an allocation of its own would fail without it
+ *    (abcore_stats.device_bytes counts it).
  */
 #ifndef ABCORE_H
 #define ABCORE_H
@@ -182,7 +185,8 @@ int abcore_community(abcore_ctx *ctx, int32_t layer, int32_t id, int32_t alpha, 
  * as one chain of increasing beta, each core seeded from the one containing it). Pair i is
  * (alphas[i], betas[i]); its masks are rows i of masks_u (n x nU, row-major) and masks_v
  * (n x nV). Results equal n separate abcore_compute calls, whatever the pair order. The
- * launch is captured once as a CUDA graph per pair list and replayed on later calls.
+ * launch is captured once as a CUDA graph per pair list and replayed on later calls, into
+ * whatever buffers they pass.
  * Errors: as abcore_compute. */
 int abcore_compute_batch(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32_t *betas,
                          uint8_t *masks_u, uint8_t *masks_v, uint32_t flags);

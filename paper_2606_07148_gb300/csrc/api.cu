@@ -50,11 +50,13 @@ int abcore_create(abcore_ctx **out, int device, void *cuda_stream) {
     if (!ctx) return ABCORE_ENOMEM;
     ctx->device = device;
     if (const char *lv = getenv("ABCORE_LOG")) ctx->prm.log_level = std::max(0, std::min(2, atoi(lv)));
-    if (cudaSetDevice(device) != cudaSuccess ||
+    size_t free_b = 0, total_b = 0;
+    if (cudaSetDevice(device) != cudaSuccess || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
         cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
         delete ctx;
         return ABCORE_ECUDA;
     }
+    ctx->spare_limit = (int64_t)(total_b / 64);
     if (cuda_stream) {
         ctx->stream = (cudaStream_t)cuda_stream;
     } else {
@@ -74,8 +76,7 @@ int abcore_destroy(abcore_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     drop_derived(ctx);
     free_graph(ctx);
-    for (auto &p : ctx->alloc_sizes) cudaFree(p.first);
-    ctx->alloc_sizes.clear();
+    ctx->free_all();
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
     return ABCORE_OK;

@@ -227,9 +227,11 @@ __global__ void __launch_bounds__(256) k_batch_emit(const int32_t *__restrict__ 
                                                     const uint8_t *__restrict__ lvl, int32_t lvl_stride,
                                                     const ChainDev *__restrict__ chains, int32_t nchains,
                                                     const PairRef *__restrict__ pairs, const int32_t *__restrict__ pidx,
-                                                    int32_t npairs, uint8_t *__restrict__ masks_u,
-                                                    uint8_t *__restrict__ masks_v) {
+                                                    int32_t npairs, uint8_t *const *__restrict__ out) {
     extern __shared__ int32_t sh[];
+    // the masks' addresses are read here, not captured, so one plan serves whatever buffers a call brings
+    uint8_t *__restrict__ const masks_u = out[0];
+    uint8_t *__restrict__ const masks_v = out[1];
     int32_t *pU0 = sh, *col = sh + nchains;
     int32_t *pc = sh + 2 * nchains, *ps = pc + npairs, *pi = ps + npairs, *pv = pi + npairs;
     for (int i = threadIdx.x; i < nchains; i += blockDim.x) {
@@ -305,7 +307,6 @@ struct Wave {
 struct BatchState {
     // key of the captured graph
     std::vector<int32_t> key_a, key_b;
-    uint8_t *key_mu = nullptr, *key_mv = nullptr;
     int64_t key_graph_n = -1, key_graph_m = -1;
     int key_chunk = 0;
     // plan
@@ -323,6 +324,8 @@ struct BatchState {
     int lvl_stride = 0;
     uint32_t *flags = nullptr;          // [grid * 32] per-block queue-closed flags (epochs)
     PeelCtl *ctl_host = nullptr;        // pinned: [waves x MAX_CHAINS_PER_WAVE]
+    uint8_t **d_out = nullptr;          // where the call's masks go: {masks_u, masks_v}
+    uint8_t **h_out = nullptr;          // pinned: its upload
     long long qcap = 0;
     bool q_dirty = false;
     cudaGraph_t graph = nullptr;
@@ -347,8 +350,7 @@ static void destroy_plan(abcore_ctx *ctx, BatchState *b) {
     ctx->release(b->d_pvs);
     ctx->release(b->d_fracs);
     ctx->release(b->prof);
-    if (b->ctl_host) cudaFreeHost(b->ctl_host);
-    b->ctl_host = nullptr;
+    ctx->host_release(b->ctl_host);
     b->key_a.clear();
     b->key_b.clear();
     b->key_graph_n = -1;
@@ -370,6 +372,8 @@ void free_batch(abcore_ctx *ctx) {
     ctx->release(b->d_mem);
     ctx->release(b->lvl);
     ctx->release(b->flags);
+    ctx->release(b->d_out);
+    ctx->host_release(b->h_out);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
     delete b;
@@ -525,7 +529,7 @@ static int make_plan(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t *a
             ABC_CU(cudaMemcpy(w.d_pidx, w.pidx.data(), sizeof(int32_t) * w.pidx.size(), cudaMemcpyHostToDevice));
         }
     }
-    ABC_CU(cudaMallocHost(&b->ctl_host, sizeof(PeelCtl) * MAX_CHAINS_PER_WAVE * b->waves.size()));
+    ABC_TRY(ctx->host_alloc(&b->ctl_host, MAX_CHAINS_PER_WAVE * b->waves.size(), "batch control readback"));
     if (ctx->prm.log_level >= 2)
         ABC_TRY(ctx->alloc(&b->prof, b->waves.size() * MAX_CHAINS_PER_WAVE * PROF_STRIDE, "batch timeline"));
     ctx->log(1, "batch plan: %d pairs, %d chains in %d waves of up to %d, grid %d blocks, %d seeded chains", n, C,
@@ -589,7 +593,7 @@ static int ensure_memory(abcore_ctx *ctx, BatchState *b, int want_chains) {
 }
 
 // Enqueue the whole batch on the stream (captured into a graph on first use).
-static int enqueue_batch(abcore_ctx *ctx, BatchState *b, uint8_t *d_mu, uint8_t *d_mv) {
+static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
     const Graph &g = ctx->g;
     const int64_t n = g.n();
     if (b->lvl_global) ABC_CU(cudaMemsetAsync(b->lvl, 0xff, (size_t)n * b->lvl_stride, ctx->stream));
@@ -646,7 +650,7 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b, uint8_t *d_mu, uint8_t 
                 ABC_CU(cudaFuncSetAttribute(k_batch_emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
             const int eg = (int)std::min<int64_t>((n + 255) / 256, (int64_t)ctx->num_sms * 8);
             k_batch_emit<<<std::max(eg, 1), 256, shm, ctx->stream>>>(g.old2new, g.nU, g.nV, b->lvl, b->lvl_stride,
-                                                                     w.d_chains, cw, w.d_pairs, w.d_pidx, np, d_mu, d_mv);
+                                                                     w.d_chains, cw, w.d_pairs, w.d_pidx, np, b->d_out);
             ctx->stats.launches++;
         }
         for (int c = 0; c < cw; ++c)
@@ -661,7 +665,9 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
     const Graph &g = ctx->g;
     if (!ctx->batch) ctx->batch = new BatchState();
     BatchState *b = ctx->batch;
-    const bool same = b->exec && b->key_mu == d_masks_u && b->key_mv == d_masks_v && b->key_graph_n == g.n() &&
+    if (!b->d_out) ABC_TRY(ctx->alloc(&b->d_out, 2, "batch mask addresses"));
+    if (!b->h_out) ABC_TRY(ctx->host_alloc(&b->h_out, 2, "batch mask addresses"));
+    const bool same = b->exec && b->key_graph_n == g.n() &&
                       b->key_graph_m == g.m && b->key_chunk == ctx->prm.chunk &&
                       b->key_a == std::vector<int32_t>(alphas, alphas + n) &&
                       b->key_b == std::vector<int32_t>(betas, betas + n);
@@ -680,8 +686,6 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
         }
         b->key_a.assign(alphas, alphas + n);
         b->key_b.assign(betas, betas + n);
-        b->key_mu = d_masks_u;
-        b->key_mv = d_masks_v;
         b->key_graph_n = g.n();
         b->key_graph_m = g.m;
         b->key_chunk = ctx->prm.chunk;
@@ -691,7 +695,7 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
             if (cs == cudaStreamCaptureStatusNone &&
                 cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
                 const int64_t l0 = ctx->stats.launches;
-                int rc = enqueue_batch(ctx, b, d_masks_u, d_masks_v);
+                int rc = enqueue_batch(ctx, b);
                 cudaGraph_t graph = nullptr;
                 cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
                 ctx->stats.launches = l0;
@@ -714,6 +718,10 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
         for (auto &m : b->mem) ABC_CU(cudaMemsetAsync(m.q, 0xff, sizeof(unsigned long long) * (size_t)b->qcap, ctx->stream));
         b->q_dirty = false;
     }
+    // (the previous call has ended: its upload is done)
+    b->h_out[0] = d_masks_u;
+    b->h_out[1] = d_masks_v;
+    ABC_CU(cudaMemcpyAsync(b->d_out, b->h_out, 2 * sizeof(uint8_t *), cudaMemcpyHostToDevice, ctx->stream));
     const bool timed = ctx->prm.timing != 0;
     if (timed) {
         if (!b->ev0) ABC_CU(cudaEventCreate(&b->ev0));
@@ -724,7 +732,7 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
         ABC_CU(cudaGraphLaunch(b->exec, ctx->stream));
         for (auto &w : b->waves) ctx->stats.launches += 1 + (w.pairs.empty() ? 0 : 1);
     } else {
-        ABC_TRY(enqueue_batch(ctx, b, d_masks_u, d_masks_v));
+        ABC_TRY(enqueue_batch(ctx, b));
     }
     // pairs of small alpha are peeled one at a time by the single peel, always the plain one (the
     // batch stays index-free): there a chain would walk far more rows than the separate peels,

@@ -526,7 +526,7 @@ int peel_prepare(abcore_ctx *ctx) {
     ABC_TRY(ctx->alloc(&w.flags, (size_t)w.flag_blocks * 32, "queue close flags"));
     ABC_CU(cudaMemsetAsync(w.flags, 0, sizeof(uint32_t) * (size_t)w.flag_blocks * 32, ctx->stream));
     w.epoch = 0;
-    ABC_CU(cudaMallocHost(&w.ctl_host, sizeof(PeelCtl) * CTL_RING));
+    ABC_TRY(ctx->host_alloc(&w.ctl_host, CTL_RING, "peel control readback"));
     for (int i = 0; i < CTL_RING; ++i) w.pending[i] = false;
     w.next = 0;
     w.last = -1;
@@ -549,8 +549,8 @@ void free_peel(abcore_ctx *ctx) {
     ctx->release(w.flags);
     ctx->release(w.trace);
     w.flag_blocks = 0;
-    if (w.ctl_host) cudaFreeHost(w.ctl_host);
-    w.ctl_host = nullptr;
+    if (w.ctl_host) cudaStreamSynchronize(ctx->stream);  // (a readback may be on its way)
+    ctx->host_release(w.ctl_host);
     for (int i = 0; i < CTL_RING; ++i) {
         w.pending[i] = false;
         for (int k = 0; k < 4; ++k)

@@ -894,6 +894,7 @@ static int grow_pools(abcore_ctx *ctx, ServeState *s) {
         const int rc = ctx->alloc(&np, (size_t)ncap, "serve inserted pool");
         if (rc) return ctx->fail(rc, "serve: target %d's inserted-edge pool cannot grow to %lld entries; its "
                                      "requests wait until device memory frees up", t, (long long)ncap);
+        ABC_CU(cudaStreamSynchronize(ctx->stream));  // (the block may be a spare one that stream used)
         ABC_CU(cudaMemcpyAsync(np, T.pool, sizeof(int32_t) * (size_t)std::max(top, 0), cudaMemcpyDeviceToDevice,
                                s->stream));
         ABC_CU(cudaStreamSynchronize(s->stream));
@@ -934,14 +935,10 @@ static void release_serve(abcore_ctx *ctx, ServeState *s) {
     ctx->release(s->d_grow);
     ctx->release(s->d_comp);
     ctx->release(s->d_comp_stale);
-    if (s->h_req) cudaFreeHost(s->h_req);
-    if (s->h_resp) cudaFreeHost(s->h_resp);
-    if (s->h_resp_seq) cudaFreeHost(s->h_resp_seq);
-    if (s->h_ctl) cudaFreeHost(s->h_ctl);
-    s->h_req = nullptr;
-    s->h_resp = nullptr;
-    s->h_resp_seq = nullptr;
-    s->h_ctl = nullptr;
+    ctx->host_release(s->h_req);
+    ctx->host_release(s->h_resp);
+    ctx->host_release(s->h_resp_seq);
+    ctx->host_release(s->h_ctl);
     if (s->loop_done) cudaEventDestroy(s->loop_done);
     s->loop_done = nullptr;
     if (s->stream) cudaStreamDestroy(s->stream);
@@ -1053,10 +1050,10 @@ int serve_start(abcore_ctx *ctx, const int32_t *ta, const int32_t *tb, int32_t n
     s->pool_cap = std::min<int64_t>(8 * std::max<int64_t>(slots, ctx->prm.serve_inserts) + 1024, INT32_MAX);
     ABC_CU(cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking));
     ABC_CU(cudaEventCreateWithFlags(&s->loop_done, cudaEventDisableTiming));
-    ABC_CU(cudaHostAlloc(&s->h_req, sizeof(abcore_req) * slots, cudaHostAllocMapped));
-    ABC_CU(cudaHostAlloc(&s->h_resp, sizeof(abcore_resp) * slots, cudaHostAllocMapped));
-    ABC_CU(cudaHostAlloc(&s->h_resp_seq, sizeof(unsigned long long) * slots, cudaHostAllocMapped));
-    ABC_CU(cudaHostAlloc(&s->h_ctl, sizeof(unsigned long long) * (16 + nt), cudaHostAllocMapped));
+    ABC_TRY(ctx->host_alloc(&s->h_req, slots, "serve request ring"));
+    ABC_TRY(ctx->host_alloc(&s->h_resp, slots, "serve response ring"));
+    ABC_TRY(ctx->host_alloc(&s->h_resp_seq, slots, "serve response ring"));
+    ABC_TRY(ctx->host_alloc(&s->h_ctl, 16 + nt, "serve control words"));
     memset(s->h_resp_seq, 0, sizeof(unsigned long long) * slots);
     memset(s->h_ctl, 0, sizeof(unsigned long long) * (16 + nt));
     ABC_CU(cudaHostGetDevicePointer((void **)&s->d_req, s->h_req, 0));
