@@ -112,14 +112,12 @@ struct PeelArgs {
     // count; dead_own then makes a crossing check the vertex's own lvl column first, so a vertex
     // queued that way is never queued twice
     int32_t dead_own, seed_col;
-    int32_t *corev;          // if set, a vertex queued during `step` gets corev[vertex] = step
     // round0: the count init lists its violators in l0 (not the queue); k_round0 walks their rows
     // with atomics that return nothing, and the scan then queues every other candidate below its
     // bound (see peel.cu)
     // (an entry is {first adjacency index, row length | L0_UPPER for a U row})
     int32_t round0;
     longlong2 *l0;
-    unsigned long long *removed;  // if set, counts the vertices queued
     // if set: a bitmap over caller ids (bit layer base + caller id) of the candidates this peel
     // removes, set when the cascade takes a fallen vertex's first chunk (round0: when the count
     // init lists it) and read, then cleared, by the caller-order mask gather

@@ -220,11 +220,6 @@ __device__ __forceinline__ void push_add(const PeelArgs &a, PushBuf<CAP> &pb, in
             uint8_t *l = a.lvl + (size_t)y * a.lvl_stride + a.lvl_col;
             if (*l == 0xFF) *l = (uint8_t)a.step;
         }
-        if (a.corev) a.corev[y] = a.step;
-    }
-    if (a.removed) {
-        const unsigned fm = __ballot_sync(ABC_FULL, want && fallen);
-        if (fm && (threadIdx.x & 31) == 0) atomicAdd(a.removed, (unsigned long long)__popc(fm));
     }
     const bool keep = want && nch > 0;
     const unsigned pm = __ballot_sync(ABC_FULL, keep);
@@ -685,13 +680,7 @@ __device__ __forceinline__ int cascade_loop(const PeelArgs &a, WarpSmem &sm, Lan
 
 // Bounded barrier over the `G` blocks of one group (a batch chain, or a whole launch). The last block to arrive can run `fixup`
 // while every other block of the group waits. Returns false if the group saw an error.
-//
-// With `watch`, the last block to arrive also records whether *watch has reached `limit` in
-// bar[16], which every block can read once the barrier has passed (it changes only at the next
-// such barrier, so all blocks read the same value).
-__device__ __forceinline__ bool group_barrier(unsigned *bar, int G, PeelCtl *ctl, bool fixup, unsigned long long timeout_ns,
-                                              const unsigned long long *watch = nullptr,
-                                              unsigned long long limit = 0) {
+__device__ __forceinline__ bool group_barrier(unsigned *bar, int G, PeelCtl *ctl, bool fixup, unsigned long long timeout_ns) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -702,7 +691,6 @@ __device__ __forceinline__ bool group_barrier(unsigned *bar, int G, PeelCtl *ctl
         const unsigned arrived = atomicAdd(bar, 1u);
         if (arrived == (unsigned)G - 1) {
             atomicExch(bar, 0u);
-            if (watch) bar[16] = ld_relaxed(watch) >= limit ? 1u : 0u;
             if (fixup) {
                 // the cascade closed the queue: every reserved slot [0, tail) was processed and
                 // emptied by its consumer, and the tickets it voided, [tail, old head), were never
