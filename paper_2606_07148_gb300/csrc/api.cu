@@ -491,8 +491,7 @@ int abcore_set_param(abcore_ctx *ctx, const char *name, int64_t value) {
         ABC_TRY(abcore_sync(ctx));
         p.round0_variant = (int)value;
     } else if (k == "round0_hub") {
-        // two layers' tables of ints in one block's shared memory (at most 227 KB)
-        if (value < 0 || value > 28672) return ctx->fail(ABCORE_EINVAL, "round0_hub must be 0..28672");
+        if (value < 0 || value > ROUND0_HUB_MAX) return ctx->fail(ABCORE_EINVAL, "round0_hub must be 0..28672");
         ABC_TRY(abcore_sync(ctx));
         p.round0_hub = (int)value;
     } else if (k == "pdl") {
@@ -569,6 +568,9 @@ int abcore_set_param(abcore_ctx *ctx, const char *name, int64_t value) {
     } else if (k == "serve_inserts") {
         if (value < 1 || value > (1 << 29)) return ctx->fail(ABCORE_EINVAL, "serve_inserts must be in [1, 2^29]");
         p.serve_inserts = value;
+    } else if (k == "small_peel") {
+        if (value < 0 || value > 1) return ctx->fail(ABCORE_EINVAL, "small_peel must be 0 or 1");
+        p.small_peel = (int)value;
     } else if (k == "log_level") {
         if (value < 0 || value > 2) return ctx->fail(ABCORE_EINVAL, "log_level must be 0..2");
         p.log_level = (int)value;
@@ -625,6 +627,7 @@ int abcore_get_param(abcore_ctx *ctx, const char *name, int64_t *value) {
     else if (k == "batch_seed") *value = p.batch_seed;
     else if (k == "batch_plain_below") *value = p.batch_plain_below;
     else if (k == "log_level") *value = p.log_level;
+    else if (k == "small_peel") *value = p.small_peel;
     else return ctx->fail(ABCORE_EINVAL, "unknown parameter '%s'", name);
     return ABCORE_OK;
 }

@@ -24,6 +24,7 @@
 #include "device.cuh"
 #include "internal.h"
 #include "peel_core.cuh"
+#include "small_peel.cuh"
 
 namespace {
 
@@ -216,6 +217,16 @@ out:
     }
 }
 
+// A batch of a small graph: one block per pair (small_peel.cuh). What each did goes to the host.
+__global__ void __launch_bounds__(abc::SMALL_THREADS, 1) k_batch_small(abc::SmallGraph G, const abc::SmallQuery *__restrict__ queries,
+                                                                       uint8_t *masks_u, uint8_t *masks_v, abc::SmallStats *host) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ abc::SmallStats st;
+    const int p = blockIdx.x;
+    abc::small_peel(G, queries[p], smem, masks_u + (size_t)p * G.nU, masks_v + (size_t)p * G.nV, &st);
+    if (threadIdx.x == 0) host[p] = st;
+}
+
 struct PairRef {
     int32_t chain;  // index into the wave's chains
     int32_t step;
@@ -326,6 +337,10 @@ struct BatchState {
     PeelCtl *ctl_host = nullptr;        // pinned: [waves x MAX_CHAINS_PER_WAVE]
     uint8_t **d_out = nullptr;          // where the call's masks go: {masks_u, masks_v}
     uint8_t **h_out = nullptr;          // pinned: its upload
+    // a small graph's batch: queries (device, and their pinned upload) and what each did (pinned)
+    abc::SmallQuery *d_queries = nullptr, *h_queries = nullptr;
+    abc::SmallStats *h_small = nullptr;
+    int32_t small_cap = 0;
     long long qcap = 0;
     bool q_dirty = false;
     cudaGraph_t graph = nullptr;
@@ -374,6 +389,9 @@ void free_batch(abcore_ctx *ctx) {
     ctx->release(b->flags);
     ctx->release(b->d_out);
     ctx->host_release(b->h_out);
+    ctx->release(b->d_queries);
+    ctx->host_release(b->h_queries);
+    ctx->host_release(b->h_small);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
     delete b;
@@ -660,11 +678,67 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
     return ABCORE_OK;
 }
 
+// Largest graph whose batch runs a block per pair: every pair's candidates fit a block, and peeling a pair by itself on one
+// SM takes less than a chain's steps on their share of the GPU (three group barriers and a cascade's
+// start and end each, about 25 us whatever their size). 8 x 8 pairs: 3,500 vertices and 20k edges 84 us against 957
+// in chains; 15,010 and 200k 115 against 1,109; 35,000 and 800k 182 against 1,119; 21,000 and 1M 134 against 810.
+constexpr int64_t SMALL_BATCH_EDGES = 1 << 20;
+static bool small_batch(const abcore_ctx *ctx) {
+    const Params &p = ctx->prm;
+    return p.small_peel && ctx->g.n() <= abc::SMALL_MAX && ctx->g.m <= SMALL_BATCH_EDGES && p.timing == 0 && p.log_level < 2 &&
+           p.batch_plain_below == 0 && p.batch_seed == 0;
+}
+
+static int batch_small(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t *alphas, const int32_t *betas, uint8_t *d_masks_u,
+                       uint8_t *d_masks_v) {
+    const Graph &g = ctx->g;
+    if (b->small_cap < n) {
+        ctx->release(b->d_queries);
+        ctx->host_release(b->h_queries);
+        ctx->host_release(b->h_small);
+        b->small_cap = 0;
+        ABC_TRY(ctx->alloc(&b->d_queries, (size_t)n, "batch queries"));
+        ABC_TRY(ctx->host_alloc(&b->h_queries, (size_t)n, "batch queries"));
+        ABC_TRY(ctx->host_alloc(&b->h_small, (size_t)n, "batch statistics"));
+        b->small_cap = n;
+    }
+    int64_t most = 0;
+    for (int32_t i = 0; i < n; ++i) {
+        const int32_t pU = (int32_t)cnt_ge(g.cntU_ge, alphas[i]), pV = (int32_t)cnt_ge(g.cntV_ge, betas[i]);
+        b->h_queries[i] = {alphas[i], betas[i], pU, pV, 0, 0};
+        most = std::max<int64_t>(most, (int64_t)pU + pV);
+    }
+    const size_t smem = abc::small_smem(most);
+    // (the largest: the limit belongs to the function, which other contexts launch too)
+    ABC_CU(cudaFuncSetAttribute(k_batch_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)abc::small_smem(abc::SMALL_MAX)));
+    ABC_CU(cudaMemcpyAsync(b->d_queries, b->h_queries, sizeof(abc::SmallQuery) * n, cudaMemcpyHostToDevice, ctx->stream));
+    k_batch_small<<<n, abc::SMALL_THREADS, smem, ctx->stream>>>({g.off, g.adj, g.old2new, g.nU, g.nV}, b->d_queries, d_masks_u, d_masks_v,
+                                                                b->h_small);
+    ABC_CU(cudaGetLastError());
+    ABC_CU(cudaStreamSynchronize(ctx->stream));
+    abcore_stats &s = ctx->stats;
+    s.launches++;
+    for (int32_t i = 0; i < n; ++i) {
+        const abc::SmallStats &t = b->h_small[i];
+        s.peels++;
+        s.candidates += (int64_t)t.inits;
+        s.init_vertices += (int64_t)t.inits;
+        s.search_probes += (int64_t)t.probes;
+        s.entries += (int64_t)t.entries;
+        s.decrements += (int64_t)t.decs;
+        s.pushes += (int64_t)t.pushes;
+        s.items += (int64_t)t.pushes;
+    }
+    s.emit_gathered += (int64_t)n * g.n();
+    return ABCORE_OK;
+}
+
 int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32_t *betas, uint8_t *d_masks_u,
                   uint8_t *d_masks_v, bool sync_and_check) {
     const Graph &g = ctx->g;
     if (!ctx->batch) ctx->batch = new BatchState();
     BatchState *b = ctx->batch;
+    if (small_batch(ctx)) return batch_small(ctx, b, n, alphas, betas, d_masks_u, d_masks_v);
     if (!b->d_out) ABC_TRY(ctx->alloc(&b->d_out, 2, "batch mask addresses"));
     if (!b->h_out) ABC_TRY(ctx->host_alloc(&b->h_out, 2, "batch mask addresses"));
     const bool same = b->exec && b->key_graph_n == g.n() &&

@@ -1212,8 +1212,9 @@ static int edges_into_rows(abcore_ctx *ctx, Graph &g, int32_t nU, int32_t nV, in
             const size_t group_smem = (size_t)SPLIT_TILE * 10 + ((size_t)12 << shift);
             const unsigned tiles = (unsigned)((m + SPLIT_TILE - 1) / SPLIT_TILE);
             uint64_t *a2 = ka, *b2 = kb, *t2 = (uint64_t *)g.adj;
-            cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem);
-            cudaFuncSetAttribute(k_regroup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)group_smem);
+            // (the largest either uses: the limit belongs to the function, which other contexts launch too)
+            cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize, SPLIT_TILE * 10 + SPLIT_BINS * 16);
+            cudaFuncSetAttribute(k_regroup, cudaFuncAttributeMaxDynamicSharedMemorySize, SPLIT_TILE * 10 + SPLIT_BINS * 12);
             // (one layer alone goes to ka, so that kb is free for its second move)
             k_split<<<tiles, SPLIT_THREADS, split_smem, ctx->stream>>>(d_eu, d_ev, m, nU, B, ngroups, whole[0] ? nullptr : a2,
                                                                        whole[1] ? nullptr : whole[0] ? a2 : b2);

@@ -183,6 +183,7 @@ struct Params {
                                // batch's per-step timeline (initial value from ABCORE_LOG)
     int query_scope = 0;       // abcore_query_edge: 0 the certificate scope (serving loop), 1 the
                                // paper's scope -- the endpoints' components re-peeled from scratch
+    int small_peel = 1;        // queries and batches of small graphs run a block per query (small_peel.cuh)
     int algo = 0;              // abcore_compute: 0 GCC+ when core numbers are prepared and it has
                                // fewer vertices to peel, else GCC; 1 always GCC; 2 always GCC+
                                // (prepares core numbers on first use)
@@ -205,6 +206,8 @@ struct Graph {
     std::vector<int64_t> cntU_ge, edgesU_ge, cntV_ge, edgesV_ge;
     int64_t n() const { return (int64_t)nU + nV; }
 };
+
+constexpr int ROUND0_HUB_MAX = 28672;  // "round0_hub": two layers' tables of ints in one block's shared memory
 
 constexpr int CTL_RING = 64;  // peels that may be in flight (ABCORE_ASYNC) before a forced wait
 
@@ -274,7 +277,8 @@ struct abcore_ctx {
     int scan_blocks = 0;     // resident k_scan blocks
     int expand_blocks = 0;   // resident k_expand blocks
     int gather_blocks = 0;   // resident k_gather blocks
-    size_t hub_smem = 0;     // dynamic shared memory k_round0_hub has been allowed so far
+    bool hub_allowed = false;    // k_round0_hub has been allowed its largest shared memory
+    bool small_allowed = false;  // ... and k_small
     BatchState *batch = nullptr;
     ServeState *serve = nullptr;
     GfqState *gfq = nullptr;   // on-the-fly queries with the component scope (query_scope = 1)

@@ -32,11 +32,18 @@
 #include "device.cuh"
 #include "internal.h"
 #include "peel_core.cuh"
+#include "small_peel.cuh"
 
 namespace {
 
 using abc::LaneStats;
 using abc::WarpSmem;
+
+// Largest graph and query k_small takes (see small_query): vertices, and entries of the candidates' rows. Whole calls,
+// one block against the general peel, with (2,3) / (10,20) / (60,60): 3,500 vertices and 20k edges 21 / 32 / 20 us
+// against 46 / 80 / 36; 15,010 and 200k 34 / 51 / 52 against 46 / 67 / 67; 30,000 and 400k 48 / 71 / 100 against
+// 46 / 55 / 164; 21,000 and 1M 46 / 46 / 95 against 33 / 46 / 83.
+constexpr int64_t SMALL_QUERY_VERTICES = 1 << 14, SMALL_QUERY_ENTRIES = 1 << 19;
 
 constexpr int INIT_THREADS = 256;
 constexpr int STREAM_THREADS = 256;
@@ -477,6 +484,25 @@ __global__ void __launch_bounds__(256) k_expand(PeelArgs a) {
     }
 }
 
+// The whole query in one block (small_peel.cuh). Its control block goes straight to the host's readback copy:
+// this kernel has no bounded wait that could fail.
+__global__ void __launch_bounds__(abc::SMALL_THREADS, 1) k_small(abc::SmallGraph G, abc::SmallQuery Q, uint8_t *mask_u, uint8_t *mask_v,
+                                                                 PeelCtl *host) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ abc::SmallStats st;
+    abc::small_peel(G, Q, smem, mask_u, mask_v, &st);
+    if (threadIdx.x < 12) {
+        const int k = threadIdx.x;
+        host->st[k] = k == ST_INIT ? st.inits : k == ST_PROBES ? st.probes : k == ST_ENTRIES ? st.entries : k == ST_DECS ? st.decs
+                    : k == ST_PUSHES || k == ST_ITEMS ? st.pushes : 0ull;
+        if (k < 4) host->ph[k] = 0;
+        if (k == 0) {
+            host->err = 0;
+            host->l0n = 0;
+        }
+    }
+}
+
 // Test hook: reserve queue slots that nothing will fill, so the consumers' bounded wait expires.
 __global__ void k_stall(PeelCtl *ctl, long long qcap, int n) {
     if (ctl->tail + (unsigned long long)n <= (unsigned long long)qcap) atomicAdd(&ctl->tail, (unsigned long long)n);
@@ -631,6 +657,18 @@ bool prefer_pruned(const abcore_ctx *ctx, int32_t alpha, int32_t beta) {
     return unc <= plain;
 }
 
+static_assert(SMALL_QUERY_VERTICES <= abc::SMALL_MAX, "every candidate has its place in the block");
+
+// Whether a query runs in one block: one SM gets through the candidates and their rows in less than the
+// time the general peel's launches and levels take, and nothing that only the general peel has is asked
+// for (a set counting mode or first round, timed kernels, the queue trace, the stall hook).
+static bool small_query(const abcore_ctx *ctx, int64_t entries, const uint8_t *mu, const uint8_t *mv) {
+    const Params &p = ctx->prm;
+    return p.small_peel && entries <= SMALL_QUERY_ENTRIES && ctx->g.n() <= SMALL_QUERY_VERTICES &&
+           p.mode < 0 && p.round0 == 0 && p.timing == 0 && p.log_level < 2 && p.debug_stall_slots == 0 &&
+           (mu != nullptr || ctx->g.nU == 0) && (mv != nullptr || ctx->g.nV == 0);
+}
+
 int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u, uint8_t *d_mask_v,
                  bool sync_and_check, bool pruned) {
     // pruned (Algorithm 2, GCC+): the core-ordered graph; with dl = min(alpha, beta) and
@@ -648,6 +686,35 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     const int32_t cU = pruned ? (int32_t)cnt_ge(ctx->pr.coreU_ge, dq) : 0;
     const int32_t cV = pruned ? (int32_t)cnt_ge(ctx->pr.coreV_ge, dq) : 0;
     const int64_t P = (int64_t)pU + pV, Pu = (int64_t)(pU - cU) + (pV - cV);
+    if (small_query(ctx, cnt_ge(ctx->g.edgesU_ge, alpha) + cnt_ge(ctx->g.edgesV_ge, beta), d_mask_u, d_mask_v)) {
+        const int slot = w.next;
+        if (w.pending[slot]) ABC_TRY(peel_finish(ctx));
+        w.next = (w.next + 1) % CTL_RING;
+        SlotInfo &si = w.info[slot];
+        si = SlotInfo{};
+        si.cands = Pu;
+        si.n = n;
+        si.emit = 1;
+        si.alpha = alpha;
+        si.beta = beta;
+        const size_t smem = abc::small_smem(Pu);
+        // (always the largest: the limit belongs to the function, which other contexts launch too)
+        if (!ctx->small_allowed) {
+            ABC_CU(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)abc::small_smem(abc::SMALL_MAX)));
+            ctx->small_allowed = true;
+        }
+        const abc::SmallGraph G{g.off, g.adj, g.old2new, nU, nV};
+        const abc::SmallQuery Q{alpha, beta, pU, pV, cU, cV};
+        k_small<<<1, abc::SMALL_THREADS, smem, ctx->stream>>>(G, Q, d_mask_u, d_mask_v, w.ctl_host + slot);
+        ABC_CU(cudaGetLastError());
+        ctx->stats.launches++;
+        ctx->stats.mode = 3;
+        ctx->stats.grid_blocks = 1;
+        w.pending[slot] = true;
+        w.last = slot;
+        ctx->pending_async = true;
+        return sync_and_check ? peel_finish(ctx) : ABCORE_OK;
+    }
     const int mode = pruned ? 3 : pick_mode(ctx, alpha, beta, pU, pV);
 
     const int slot = w.next;
@@ -789,9 +856,10 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
                     const int hU = (int)std::min<int64_t>(pU, ctx->prm.round0_hub);
                     const int hV = (int)std::min<int64_t>(pV, ctx->prm.round0_hub);
                     const size_t smem = (size_t)(hU + hV) * sizeof(int);
-                    if (ctx->hub_smem < smem) {
-                        ABC_CU(cudaFuncSetAttribute(k_round0_hub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                        ctx->hub_smem = smem;
+                    if (!ctx->hub_allowed) {  // (the largest table, as for k_small)
+                        ABC_CU(cudaFuncSetAttribute(k_round0_hub, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    2 * ROUND0_HUB_MAX * (int)sizeof(int)));
+                        ctx->hub_allowed = true;
                     }
                     ABC_CU(launch_k(pdl && prev_k, k_round0_hub, std::min<int64_t>(gr, ctx->num_sms), 1024,
                                     ctx->stream, smem, a, hU, hV));
