@@ -330,7 +330,7 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "local_rounds" [256] batches a warp may chain on its own pushes (0..4096).
  *   "flush_steps"* [4]  steps a buffered push may wait before its warp flushes.
  * Batch:
- *   "batch_wave"* [4]   chains per wave (0..32; 0: all at once).
+ *   "batch_wave"* [4, 8 or 16, by the size of the graph]  chains per wave (0..32; 0: all at once).
  *   "batch_plain_below"* [0] pairs with alpha below this run as single peels, not chains.
  *   "batch_seed"* [0]   1: seed each chain from the finished chain of the next smaller alpha.
  *   "packed_counts" [1] chains keep 16-bit counts whenever every degree fits.

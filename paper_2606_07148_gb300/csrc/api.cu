@@ -617,7 +617,7 @@ int abcore_get_param(abcore_ctx *ctx, const char *name, int64_t *value) {
     else if (k == "emit_scatter_max_pct") *value = p.emit_scatter_max_pct;
     else if (k == "emit_bitmap_min_pct") *value = p.emit_bitmap_min_pct;
     else if (k == "probe_bytes") *value = (int64_t)p.probe_bytes;
-    else if (k == "batch_wave") *value = p.batch_wave;
+    else if (k == "batch_wave") *value = batch_wave_of(ctx);
     else if (k == "hub_degree") *value = p.hub_degree;
     else if (k == "timing") *value = p.timing;
     else if (k == "timing_kinds") *value = p.timing_kinds;

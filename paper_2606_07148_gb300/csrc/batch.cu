@@ -230,10 +230,16 @@ __global__ void __launch_bounds__(abc::SMALL_THREADS, 1) k_batch_small(abc::Smal
 struct PairRef {
     int32_t chain;  // index into the wave's chains
     int32_t step;
-    int32_t pv;     // V candidate prefix of the pair's beta
 };
 
-// Masks of every pair of a wave, in the caller's ids: one thread per vertex, one byte per pair.
+// Masks of every pair of a wave, in the caller's ids. With up to 16 chains (a row of lvl is WORDS 4-byte words), layers
+// that are multiples of four and aligned masks (`vec`), a thread takes four consecutive ids: their numbers
+// and removal steps come in 16-byte loads, and per pair one byte-wise comparison of the four steps gives
+// the 4-byte store. The pairs of a chain lie together (first[c] .. first[c + 1]); whether an id is a candidate of a chain
+// does not depend on the pair (a V vertex that leaves the prefix at a later step has that step recorded). Bound
+// by the masks' writes: 256 pairs on 6M vertices 1.54 GB, 0.29 ms (1.33 in four waves of four chains that
+// tested every id's prefix for every pair).
+template <int WORDS>
 __global__ void __launch_bounds__(256) k_batch_emit(const int32_t *__restrict__ old2new, int32_t nU, int32_t nV,
                                                     const uint8_t *__restrict__ lvl, int32_t lvl_stride,
                                                     const ChainDev *__restrict__ chains, int32_t nchains,
@@ -243,45 +249,65 @@ __global__ void __launch_bounds__(256) k_batch_emit(const int32_t *__restrict__ 
     // the masks' addresses are read here, not captured, so one plan serves whatever buffers a call brings
     uint8_t *__restrict__ const masks_u = out[0];
     uint8_t *__restrict__ const masks_v = out[1];
-    int32_t *pU0 = sh, *col = sh + nchains;
-    int32_t *pc = sh + 2 * nchains, *ps = pc + npairs, *pi = ps + npairs, *pv = pi + npairs;
+    int32_t *pU0 = sh, *pV0 = sh + nchains, *col = sh + 2 * nchains, *first = sh + 3 * nchains;  // (first: nchains + 1)
+    int32_t *ps = first + nchains + 1, *pi = ps + npairs;
     for (int i = threadIdx.x; i < nchains; i += blockDim.x) {
         pU0[i] = chains[i].pU0;
+        pV0[i] = chains[i].pV0;
         col[i] = chains[i].col;
     }
-    for (int i = threadIdx.x; i < npairs; i += blockDim.x) {
-        pc[i] = pairs[i].chain;
+    for (int i = threadIdx.x; i < npairs; i += blockDim.x) {  // (sorted by chain)
         ps[i] = pairs[i].step;
         pi[i] = pidx[i];
-        pv[i] = pairs[i].pv;
+        for (int c = (i ? pairs[i - 1].chain : -1) + 1; c <= pairs[i].chain; ++c) first[c] = i;
+        if (i == npairs - 1)
+            for (int c = pairs[i].chain + 1; c <= nchains; ++c) first[c] = npairs;
     }
     __syncthreads();
     const int64_t n = (int64_t)nU + nV;
-    if (lvl_stride == 4 && (nU & 3) == 0 && (nV & 3) == 0 &&
+    if (WORDS > 0 && (nU & 3) == 0 && (nV & 3) == 0 &&
         ((reinterpret_cast<uintptr_t>(masks_u) | reinterpret_cast<uintptr_t>(masks_v)) & 3) == 0) {
-        // four consecutive caller ids per thread (16-byte id load, one 4-byte store per pair), and
-        // each vertex's removal steps in one 4-byte row (at most four chains a wave)
         const int4 *o4 = reinterpret_cast<const int4 *>(old2new);
         for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n / 4; q += (int64_t)gridDim.x * blockDim.x) {
             const int64_t i = 4 * q;
             const int4 xv = __ldg(&o4[q]);
             const int32_t xs[4] = {xv.x, xv.y, xv.z, xv.w};
             const bool upper = i < nU;  // nU is a multiple of four: the quad is in one layer
-            uint32_t rows[4];
+            uint8_t *const dst = upper ? masks_u + i : masks_v + (i - nU);
+            const size_t stride = upper ? (size_t)nU : (size_t)nV;
+            uint32_t row[4][WORDS > 0 ? WORDS : 1];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) rows[j] = __ldg(reinterpret_cast<const uint32_t *>(lvl + (size_t)xs[j] * 4));
-            for (int p = 0; p < npairs; ++p) {
-                const int ch = pc[p];
-                const unsigned sh = 8u * (unsigned)col[ch];
-                uint32_t bytes = 0;
+            for (int j = 0; j < 4; ++j) {
+                const uint8_t *r = lvl + (size_t)xs[j] * (4 * WORDS);
+                if constexpr (WORDS == 4) {
+                    const uint4 w = __ldg(reinterpret_cast<const uint4 *>(r));
+                    row[j][0] = w.x;
+                    row[j][1] = w.y;
+                    row[j][2] = w.z;
+                    row[j][3] = w.w;
+                } else {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const bool cand = upper ? (xs[j] < pU0[ch]) : (xs[j] - nU < pv[p]);
-                    const bool in = cand && (int)((rows[j] >> sh) & 0xffu) > ps[p];
-                    bytes |= (in ? 1u : 0u) << (8 * j);
+                    for (int w = 0; w < WORDS; ++w) row[j][w] = __ldg(reinterpret_cast<const uint32_t *>(r) + w);
                 }
-                if (upper) *reinterpret_cast<uint32_t *>(masks_u + (size_t)pi[p] * nU + i) = bytes;
-                else *reinterpret_cast<uint32_t *>(masks_v + (size_t)pi[p] * nV + (i - nU)) = bytes;
+            }
+#pragma unroll
+            for (int w = 0; w < WORDS; ++w) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int c = 4 * w + k;  // (a wave's chains have columns 0, 1, ... in order)
+                    if (c >= nchains) break;
+                    const int p0 = first[c], p1 = first[c + 1];
+                    if (p0 == p1) continue;
+                    // the four ids' steps for this chain in one word, 0 for one that is no candidate (never above a step)
+                    const int32_t lim = upper ? pU0[c] : nU + pV0[c];
+                    uint32_t lv = 0;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) lv |= xs[j] < lim ? ((row[j][w] >> (8 * k)) & 0xffu) << (8 * j) : 0u;
+                    for (int p = p0; p < p1; ++p) {
+                        const uint32_t in = __vcmpgtu4(lv, (uint32_t)ps[p] * 0x01010101u) & 0x01010101u;
+                        __stcs(reinterpret_cast<uint32_t *>(dst + (size_t)pi[p] * stride), in);
+                    }
+                }
             }
         }
         return;
@@ -290,14 +316,13 @@ __global__ void __launch_bounds__(256) k_batch_emit(const int32_t *__restrict__ 
         const int32_t x = __ldg(&old2new[i]);
         const bool upper = i < nU;
         const uint8_t *row = lvl + (size_t)x * lvl_stride;
-        for (int p = 0; p < npairs; ++p) {
-            const int ch = pc[p];
-            // a candidate of the pair that had not fallen by its step (V vertices that left the
-            // prefix at a later step are never queued: the prefix test places them)
-            const bool cand = upper ? (x < pU0[ch]) : (x - nU < pv[p]);
-            const uint8_t v = (cand && __ldg(&row[col[ch]]) > ps[p]) ? 1 : 0;
-            if (upper) masks_u[(size_t)pi[p] * nU + i] = v;
-            else masks_v[(size_t)pi[p] * nV + (i - nU)] = v;
+        for (int c = 0; c < nchains; ++c) {
+            const int l = (upper ? x < pU0[c] : x - nU < pV0[c]) ? (int)__ldg(&row[col[c]]) : 0;
+            for (int p = first[c]; p < first[c + 1]; ++p) {
+                const uint8_t v = l > ps[p] ? 1 : 0;
+                if (upper) masks_u[(size_t)pi[p] * nU + i] = v;
+                else masks_v[(size_t)pi[p] * nV + (i - nU)] = v;
+            }
         }
     }
 }
@@ -417,6 +442,8 @@ static int ensure_lvl(abcore_ctx *ctx, BatchState *b, int stride) {
     return ctx->alloc(&b->lvl, (size_t)std::max<int64_t>(ctx->g.n(), 1) * stride, "batch levels");
 }
 
+// Counts of a wave's chains (see batch_wave_of)
+constexpr int64_t BATCH_WAVE_BYTES = 240ll << 20;
 constexpr int MAX_LVL_COLS = 64;  // chains with a column of their own in lvl (beyond: one per wave slot)
 
 // Build the plan for a pair list: chains by alpha, waves, seeds, slices, device tables.
@@ -447,7 +474,7 @@ static int make_plan(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t *a
     const int C = (int)chains.size();
     const int grid = batch_grid(ctx);
     int per_wave = std::max(1, std::min({MAX_CHAINS_PER_WAVE, grid, b->nmem}));
-    if (ctx->prm.batch_wave > 0) per_wave = std::min(per_wave, ctx->prm.batch_wave);
+    if (batch_wave_of(ctx) > 0) per_wave = std::min(per_wave, batch_wave_of(ctx));
     const int NW = (C + per_wave - 1) / per_wave;
     const bool own_cols = ctx->prm.batch_seed && C <= MAX_LVL_COLS;
     b->lvl_global = own_cols;
@@ -528,8 +555,21 @@ static int make_plan(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t *a
         }
         const auto &bs = chains[ci].betas;
         const int step = (int)(std::lower_bound(bs.begin(), bs.end(), betas[i]) - bs.begin());
-        b->waves[wave_of[ci]].pairs.push_back({slot_of[ci], step, (int32_t)cnt_ge(g.cntV_ge, betas[i])});
+        b->waves[wave_of[ci]].pairs.push_back({slot_of[ci], step});
         b->waves[wave_of[ci]].pidx.push_back(i);
+    }
+    for (auto &w : b->waves) {  // the pairs of a chain together (k_batch_emit)
+        std::vector<size_t> order(w.pairs.size());
+        for (size_t k = 0; k < order.size(); ++k) order[k] = k;
+        std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return w.pairs[x].chain < w.pairs[y].chain; });
+        std::vector<PairRef> pr;
+        std::vector<int32_t> pi;
+        for (size_t k : order) {
+            pr.push_back(w.pairs[k]);
+            pi.push_back(w.pidx[k]);
+        }
+        w.pairs.swap(pr);
+        w.pidx.swap(pi);
     }
     ABC_TRY(ctx->alloc(&b->d_betas, b->betas.size(), "batch betas"));
     ABC_CU(cudaMemcpy(b->d_betas, b->betas.data(), sizeof(int32_t) * b->betas.size(), cudaMemcpyHostToDevice));
@@ -558,6 +598,18 @@ static int make_plan(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t *a
 // Counts of the batch's chains are 16-bit when every degree fits (parameter "packed_counts").
 static bool batch_packed(const abcore_ctx *ctx) {
     return ctx->prm.packed_counts && std::max(ctx->g.maxdegU, ctx->g.maxdegV) <= 65535;
+}
+
+// Chains sharing the GPU at once, unless "batch_wave" says otherwise: more of them leave fewer blocks waiting in
+// narrow steps, until their counts no longer find room in L2. 16 chains of 6M vertices (12 MB of counts each), 256
+// pairs on 100M edges: waves of 2 / 4 / 8 / 16 34.9 / 25.0 / 21.1 / 19.6 ms; 0.6M vertices, 144 pairs on 10M edges: 9.9 / 6.4 /
+// 5.5 / 4.2; 30M vertices (60 MB each, 500M edges): 4 was the best.
+int batch_wave_of(const abcore_ctx *ctx) {
+    if (ctx->prm.batch_wave >= 0) return ctx->prm.batch_wave;
+    const int64_t bytes = (batch_packed(ctx) ? 2 : 4) * ctx->g.n();
+    int w = 16;
+    while (w > 4 && w * bytes > BATCH_WAVE_BYTES) w /= 2;
+    return w;
 }
 
 // Chain workspaces: counts, queue, control block and barrier per concurrent chain, plus lvl.
@@ -662,12 +714,16 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
         ctx->stats.launches++;
         if (!w.pairs.empty()) {
             const int np = (int)w.pairs.size();
-            const size_t shm = sizeof(int32_t) * (2 * cw + 4 * np);
+            const size_t shm = sizeof(int32_t) * (4 * cw + 1 + 2 * np);
             if (shm > 200 * 1024) return ctx->fail(ABCORE_EINVAL, "too many pairs in one batch wave");
+            // a wave whose chains have the columns 0, 1, ... of rows of at most 16
+            const int words = !b->lvl_global && b->lvl_stride <= 16 ? b->lvl_stride / 4 : 0;
+            auto *emit = words == 1 ? k_batch_emit<1> : words == 2 ? k_batch_emit<2> : words == 3 ? k_batch_emit<3>
+                       : words == 4 ? k_batch_emit<4> : k_batch_emit<0>;
             if (shm > 48 * 1024)
-                ABC_CU(cudaFuncSetAttribute(k_batch_emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+                ABC_CU(cudaFuncSetAttribute(emit, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
             const int eg = (int)std::min<int64_t>((n + 255) / 256, (int64_t)ctx->num_sms * 8);
-            k_batch_emit<<<std::max(eg, 1), 256, shm, ctx->stream>>>(g.old2new, g.nU, g.nV, b->lvl, b->lvl_stride,
+            emit<<<std::max(eg, 1), 256, shm, ctx->stream>>>(g.old2new, g.nU, g.nV, b->lvl, b->lvl_stride,
                                                                      w.d_chains, cw, w.d_pairs, w.d_pidx, np, b->d_out);
             ctx->stats.launches++;
         }
@@ -751,7 +807,7 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
         for (int32_t i = 0; i < n; ++i)
             if (alphas[i] >= ctx->prm.batch_plain_below) na[alphas[i]]++;
         int want = std::min<int>((int)na.size(), MAX_CHAINS_PER_WAVE);
-        if (ctx->prm.batch_wave > 0) want = std::min(want, ctx->prm.batch_wave);
+        if (batch_wave_of(ctx) > 0) want = std::min(want, batch_wave_of(ctx));
         if (want > 0) {
             ABC_TRY(ensure_memory(ctx, b, want));
             ABC_TRY(make_plan(ctx, b, n, alphas, betas));

@@ -170,8 +170,8 @@ struct Params {
     int batch_seed = 0;        // 1: a batch chain is seeded from the finished chain of the next
                                // smaller alpha with the same betas (its non-members are queued at
                                // once); measured no faster on the power-law grids, so off by default
-    int batch_wave = 4;        // chains sharing the GPU at once (0 = as many as fit, up to 32);
-                               // 4 measured best on a 500M-edge graph (counts stay closer to L2)
+    int batch_wave = -1;       // chains sharing the GPU at once (0 = as many as fit, up to 32; -1, until it is
+                               // set: by the size of their counts, batch_wave_of)
     int debug_stall_slots = 0; // test hook: queue slots reserved but never written
     int timing = 0;            // 1: CUDA events around each launch, summed into stats.kernel_ms
     int timing_kinds = 0xff;   // single peel: the kernel kinds (bit ABCORE_K_*) timed. An event
@@ -485,6 +485,7 @@ int cascade_grid(abcore_ctx *ctx);
 int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32_t *betas,
                   uint8_t *d_masks_u, uint8_t *d_masks_v, bool sync_and_check);
 void free_batch(abcore_ctx *ctx);
+int batch_wave_of(const abcore_ctx *ctx);  // "batch_wave", or what the loaded graph's size makes it
 
 // serve.cu
 int query_edge(abcore_ctx *ctx, int32_t u, int32_t v, int op, int32_t alpha, int32_t beta,
