@@ -309,7 +309,8 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "mode" [-1]         per-layer count init: -1 cost model, 0..3 bit 0 U by row search, bit 1 V.
  *   "hub_degree"* [256] rows of at least this degree always count by search (0: none).
  *   "probe_bytes"* [32] the cost model's price of a search probe (steers search vs stream).
- *   "round0"* [0]       1: walk the initial violators' rows with no-return decrements first.
+ *   "round0"* [by query] 1: walk the initial violators' rows with no-return decrements first; 0: queue
+ *                       them. Until it is set, queries whose first round is long take 1 (with form 4).
  *   "round0_variant"* [0] that walk's form: 0..3 lane-per-entry (entries in flight / blocks an SM:
  *                       8/any, 4/8, 16/4, 8/8), 4 four rows per warp, 5 the same in one 1024-thread
  *                       block per SM summing hub decrements in shared memory.
@@ -324,11 +325,12 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "blocks_per_sm"* [0] resident blocks an SM for the cascade and the batch (0: as many as fit;
  *                       batch: 2 selects the batch kernel compiled for two blocks an SM).
  *   "chunk"* [1024]     adjacency entries per work item (32..2^20).
- *   "grab_div"* [0]     queue items per grab = backlog / grab_div, 1..32 (0: resident warps / 8).
+ *   "grab_div"* [0]     queue items per grab = backlog / grab_div, 1..32 (0: half the resident warps, or
+ *                       all of them after a long first round).
  *   "batch_entries"* [1024] entries a warp walks per batch (128..2^24; the rest is re-queued).
  *   "batch_entries_small"* [512] the limit when a warp's grab leaves the queue nearly empty (0 off).
  *   "local_rounds" [256] batches a warp may chain on its own pushes (0..4096).
- *   "flush_steps"* [4]  steps a buffered push may wait before its warp flushes.
+ *   "flush_steps"* [16]  steps a buffered push may wait before its warp flushes.
  * Batch:
  *   "batch_wave"* [4, 8 or 16, by the size of the graph]  chains per wave (0..32; 0: all at once).
  *   "batch_plain_below"* [0] pairs with alpha below this run as single peels, not chains.

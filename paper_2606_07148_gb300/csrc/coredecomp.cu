@@ -371,6 +371,7 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
     const Graph &g = ctx->g;
     const int64_t n = std::max<int64_t>(g.n(), 1);
     ABC_TRY(peel_finish(ctx));
+    ABC_TRY(peel_prepare(ctx));  // (for the queries this is the preprocessing of)
     int32_t *words = nullptr, *tables = nullptr;
     unsigned *small = nullptr;
     PeelCtl *ctl = nullptr;

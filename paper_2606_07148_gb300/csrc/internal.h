@@ -136,14 +136,12 @@ struct Params {
     int chunk = 1024;
     int batch_entries = 1024;  // see PeelArgs (1024 kept a 94k-candidate, 18-level cascade 4.5x
                                // faster than 4096; the autotuner may raise it)
-    int flush_steps = 4;
+    int flush_steps = 16;
     int packed_counts = 1;     // batch chains keep 16-bit counts when every degree fits
-    int round0 = 0;            // single peel: walk the initial candidate violators' rows with
+    int round0 = -1;           // single peel: walk the initial candidate violators' rows with
                                // no-return atomics when a layer counts by search (k_round0), instead
-                               // of queueing them. Pays where the cascade is bound by atomic
-                               // throughput (1.5B edges, (64,64): 2.01 -> 1.74 ms); costs where it is
-                               // latency-bound (80M edges, (50,50): 0.30 -> 0.53 ms). The autotuner
-                               // decides per workload.
+                               // of queueing them; -1, until it is set: where that saves enough
+                               // (first_round_entries)
     int round0_variant = 0;    // k_round0's compiled (entries per lane per step, blocks per SM) pair:
                                // 0 (8, any), 1 (4, 8), 2 (16, 4), 3 (8, 8); 4: rows four at a time;
                                // 5: rows four at a time, hub decrements summed in shared memory
@@ -153,7 +151,7 @@ struct Params {
     int pdl = 1;               // single peel: launch the kernels after the count init as
                                // programmatic dependents of the one before (each waits for its
                                // predecessor on the device; the launch latency overlaps its tail)
-    int grab_div = 0;          // 0 = automatic (resident warps / 8)
+    int grab_div = 0;          // 0 = automatic (see peel_compute)
     int local_rounds = 256;    // single peel: see PeelArgs::local_rounds
     int batch_entries_small = 512; // single peel: see PeelArgs::batch_entries_small (0: off)
     int threads = 256;
@@ -238,7 +236,8 @@ struct PeelWork {
     bool q_dirty = false;          // queue not known to be all-empty
     uint32_t *flags = nullptr;     // [grid * 32] per-block queue-closed flags (epochs)
     int flag_blocks = 0;
-    longlong2 *l0 = nullptr;       // [n] initial candidate violators' rows (round0)
+    longlong2 *l0 = nullptr;       // [l0_cap] initial candidate violators' rows (round0)
+    int64_t l0_cap = 0;
     uint32_t *fallen = nullptr;    // [(n + 31) / 32] removed-candidate bitmap (all zero between peels)
     bool fallen_dirty = false;     // a failed peel may have left bits set
     uint32_t epoch = 0;            // last cascade epoch handed out

@@ -45,6 +45,10 @@ using abc::WarpSmem;
 // 46 / 55 / 164; 21,000 and 1M 46 / 46 / 95 against 33 / 46 / 83.
 constexpr int64_t SMALL_QUERY_VERTICES = 1 << 14, SMALL_QUERY_ENTRIES = 1 << 19;
 
+// First rounds of at least this many entries walk the initial violators' rows without returns (unless "round0" is set)
+constexpr double ROUND0_MIN_ENTRIES = 2e6;
+constexpr int SWIZZLE_MAX_PCT = 30;  // counts are spread when candidates are less than this share of the vertices
+
 constexpr int INIT_THREADS = 256;
 constexpr int STREAM_THREADS = 256;
 
@@ -434,10 +438,16 @@ __device__ __forceinline__ void k_cascade_emit(const PeelArgs &a, int ok, int64_
 // cascade failed (the next peel then clears the removal bitmap).
 __global__ void __launch_bounds__(256) k_gather(PeelArgs a) {
     abc::grid_dep_wait();
-    if (abc::ld_relaxed_i32(&a.ctl->err) != 0) return;
+    if (a.ctl != nullptr && abc::ld_relaxed_i32(&a.ctl->err) != 0) return;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     k_cascade_emit(a, 1, gw, nw, threadIdx.x & 31);
+}
+
+// The scatter (emission 2) by itself, for a query with nothing to peel.
+__global__ void __launch_bounds__(256) k_scatter(PeelArgs a) {
+    abc::grid_dep_launch();
+    k_cascade_emit(a, 1, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((int64_t)gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
 // After a scatter: both masks from the survivor bitmap, 32 caller ids (one word) per thread
@@ -532,8 +542,6 @@ int peel_prepare(abcore_ctx *ctx) {
     int64_t bv = 0;
     const int64_t slots = std::max(n, swz_layout(g.nU, g.nV, &mu, &mv, &bv));
     if (w.n == n && w.qcap >= qcap && w.cnt && w.cnt_slots >= slots && w.flag_blocks >= cascade_grid(ctx)) {
-        // the round0 list (16 bytes a vertex) is only made once round0 is asked for
-        if (ctx->prm.round0 && !w.l0) ABC_TRY(ctx->alloc(&w.l0, (size_t)std::max<int64_t>(n, 1), "initial violators"));
         return ABCORE_OK;
     }
     free_peel(ctx);
@@ -541,7 +549,6 @@ int peel_prepare(abcore_ctx *ctx) {
     ABC_TRY(ctx->alloc(&w.cnt, (size_t)std::max<int64_t>(slots, 1), "peel counts"));
     w.cnt_slots = slots;
     ABC_TRY(ctx->alloc(&w.plen, (size_t)std::max<int64_t>(n, 1), "peel prefixes"));
-    if (ctx->prm.round0) ABC_TRY(ctx->alloc(&w.l0, (size_t)std::max<int64_t>(n, 1), "initial violators"));
     ABC_TRY(ctx->alloc(&w.q, (size_t)qcap, "peel queue"));
     ABC_TRY(ctx->alloc(&w.ctl, CTL_RING, "peel control"));
     ABC_TRY(ctx->alloc(&w.stage, (size_t)std::max<int64_t>(n, 1), "mask staging"));
@@ -568,6 +575,7 @@ void free_peel(abcore_ctx *ctx) {
     ctx->release(w.cnt);
     ctx->release(w.plen);
     ctx->release(w.l0);
+    w.l0_cap = 0;
     ctx->release(w.q);
     ctx->release(w.ctl);
     ctx->release(w.stage);
@@ -615,12 +623,19 @@ cudaError_t launch_k(bool pdl, void (*k)(P...), int64_t grid, int block, cudaStr
 // search starts where the layer's share f of candidate entries puts the boundary; with the
 // binomial spread sigma = sqrt(L f (1 - f)) of a row of length L about that guess, it reads
 // about 1 + 2 log2(1 + sigma / 8) sectors (one, then a gallop and a bisection over the spread).
+// (5M edges, (2,2) / (5,5): streaming 48 / 59 us, searching 35 / 46, although it reads more; 80M edges, (2,2):
+// 112 and 126.)
+constexpr double STREAM_LAUNCHES = 5e5;
 int pick_mode(const abcore_ctx *ctx, int32_t alpha, int32_t beta, int32_t pU, int32_t pV) {
     const Graph &g = ctx->g;
     if (ctx->prm.mode >= 0) return ctx->prm.mode & 3;
     const double m = (double)std::max<int64_t>(g.m, 1);
     const double pb = ctx->prm.probe_bytes / 32.0;  // relative probe cost (default 1)
     const int hd = ctx->prm.hub_degree > 0 ? ctx->prm.hub_degree : INT32_MAX;
+    struct Cost {
+        double search, stream;
+        bool streams;
+    };
     auto layer = [&](int64_t p, int32_t thr, const std::vector<int64_t> &cnt, const std::vector<int64_t> &edges,
                      double other_violator_entries, double f) {
         // non-hub candidates: degree in [thr, hd)
@@ -629,16 +644,44 @@ int pick_mode(const abcore_ctx *ctx, int32_t alpha, int32_t beta, int32_t pU, in
         const double en = (double)(cnt_ge(edges, thr) - cnt_ge(edges, top));
         const double avg = pn > 0 ? en / pn : 1.0;
         const double sigma = std::sqrt(std::max(avg, 1.0) * f * (1.0 - f));
-        const double search = pn * (0.5 + pb * (1.0 + 2.0 * std::log2(1.0 + sigma / 8.0)));
+        Cost c;
+        c.search = pn * (0.5 + pb * (1.0 + 2.0 * std::log2(1.0 + sigma / 8.0)));
         // stream: every violator entry is read; the share landing on non-hub candidates decrements
-        const double stream = pn * 0.7 + other_violator_entries * (0.08 + 0.8 * (en / m));
-        return search <= stream;
+        c.stream = pn * 0.7 + other_violator_entries * (0.08 + 0.8 * (en / m));
+        c.streams = other_violator_entries > 0 && p > 0;
+        return c;
     };
     const double eU = (double)cnt_ge(g.edgesU_ge, alpha), eV = (double)cnt_ge(g.edgesV_ge, beta);
     // a U row's entries are V ids: the share below the bound is the V candidates' degree over m
-    const bool sU = layer(pU, alpha, g.cntU_ge, g.edgesU_ge, m - eV, eV / m);
-    const bool sV = layer(pV, beta, g.cntV_ge, g.edgesV_ge, m - eU, eU / m);
-    return (sU ? 1 : 0) | (sV ? 2 : 0);
+    const Cost cu = layer(pU, alpha, g.cntU_ge, g.edgesU_ge, m - eV, eV / m);
+    const Cost cv = layer(pV, beta, g.cntV_ge, g.edgesV_ge, m - eU, eU / m);
+    // streaming in either layer adds two launches, the stream and the scan after it
+    int best = 3;
+    double least = 0;
+    for (int k = 3; k >= 0; --k) {
+        const bool su = (k & 1) != 0, sv = (k & 2) != 0;
+        const double t = (su ? cu.search : cu.stream) + (sv ? cv.search : cv.stream) +
+                         ((!su && cu.streams) || (!sv && cv.streams) ? STREAM_LAUNCHES : 0.0);
+        if (k == 3 || t < least) {
+            best = k;
+            least = t;
+        }
+    }
+    return best;
+}
+
+// Row entries the first round is expected to walk when both layers count by search: a candidate of degree d has about
+// d f live candidate neighbours, f being the share of its layer's entries below the other layer's boundary, so
+// the initial violators are the candidates of degree below threshold / f.
+static double first_round_entries(const Graph &g, int32_t alpha, int32_t beta) {
+    const double m = (double)std::max<int64_t>(g.m, 1);
+    auto layer = [&](int32_t thr, const std::vector<int64_t> &edges, double f) {
+        if (thr <= 0 || f <= 0.0) return 0.0;
+        const double top = std::min((double)INT32_MAX, std::ceil((double)thr / f));
+        return f * (double)(cnt_ge(edges, thr) - cnt_ge(edges, (int32_t)top));
+    };
+    const double eU = (double)cnt_ge(g.edgesU_ge, alpha), eV = (double)cnt_ge(g.edgesV_ge, beta);
+    return layer(alpha, g.edgesU_ge, eV / m) + layer(beta, g.edgesV_ge, eU / m);
 }
 
 // With core numbers prepared, is the pruned peel (GCC+) the cheaper one? GCC+ initialises and
@@ -665,7 +708,7 @@ static_assert(SMALL_QUERY_VERTICES <= abc::SMALL_MAX, "every candidate has its p
 static bool small_query(const abcore_ctx *ctx, int64_t entries, const uint8_t *mu, const uint8_t *mv) {
     const Params &p = ctx->prm;
     return p.small_peel && entries <= SMALL_QUERY_ENTRIES && ctx->g.n() <= SMALL_QUERY_VERTICES &&
-           p.mode < 0 && p.round0 == 0 && p.timing == 0 && p.log_level < 2 && p.debug_stall_slots == 0 &&
+           p.mode < 0 && p.round0 <= 0 && p.timing == 0 && p.log_level < 2 && p.debug_stall_slots == 0 &&
            (mu != nullptr || ctx->g.nU == 0) && (mv != nullptr || ctx->g.nV == 0);
 }
 
@@ -726,7 +769,11 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     a.off = g.off;
     a.adj = g.adj;
     a.cnt = w.cnt;
-    set_count_layout(a, pU, pV, ctx->prm.count_swizzle != 0);
+    // Spread counts (PeelArgs::swz) where a few candidates take many decrements; with most vertices candidates, few of
+    // them fall, and the count init and the scan write and read all counts in vertex order (80M edges, vertex
+    // order against spread: (2,2) 90 / 112 us, (5,3) 120 / 132, (10,10) 154 / 152, (50,50) 276 / 256, candidates 97, 78, 53
+    // and 8 % of the vertices; 300M edges: (10,10) 597 / 638 at 35 %, (64,64) 577 / 496 at 4 %).
+    set_count_layout(a, pU, pV, ctx->prm.count_swizzle != 0 && P * 100 < n * SWIZZLE_MAX_PCT);
     a.plen = w.plen;
     a.q = w.q;
     a.qcap = w.qcap;
@@ -751,9 +798,33 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
         ABC_CU(cudaMemsetAsync(a.trace, 0, abc::TRACE_WORDS * sizeof(unsigned long long), ctx->stream));
     }
     const int blocks = cascade_grid(ctx);
-    a.grab_div = ctx->prm.grab_div > 0 ? ctx->prm.grab_div : std::max(1, blocks * (256 / 32) / 8);
     a.searchU = mode & 1;
     a.searchV = (mode >> 1) & 1;
+    // The initial violators' rows: walked first without returns, or queued. The walk and its scan cost two launches; no
+    // crossing is looked for in it, which runs half again as fast.
+    int round0 = ctx->prm.round0, round0_variant = ctx->prm.round0_variant;
+    if (round0 < 0) {
+        round0 = !pruned && mode == 3 && first_round_entries(g, alpha, beta) >= ROUND0_MIN_ENTRIES ? 1 : 0;
+        round0_variant = 4;
+    }
+    if (round0 && (a.searchU || a.searchV) && w.l0_cap < Pu) {
+        ctx->release(w.l0);
+        w.l0_cap = 0;
+        const int rc = ctx->alloc(&w.l0, (size_t)Pu, "initial violators");
+        if (rc && ctx->prm.round0 > 0) return rc;
+        if (rc == ABCORE_OK) w.l0_cap = Pu;
+        else {  // no room for the list: queue them
+            round0 = 0;
+            ctx->err.clear();
+        }
+    }
+    a.round0 = (round0 && (a.searchU || a.searchV)) ? 1 : 0;
+    // A warp's grab: its share of what is queued. With an eighth of the warps as the divisor the first warps took all of a
+    // queue of 20,000 items, 31 each, and the tickets they held beyond it drew most later items to them
+    // too (5M edges, (20,20) / (40,40): 152 / 218 us, with half the warps 71 / 81); after a long first round
+    // what is queued is little and deep, and all warps share it.
+    const int warps = blocks * (256 / 32);
+    a.grab_div = ctx->prm.grab_div > 0 ? ctx->prm.grab_div : std::max(1, a.round0 ? warps : warps / 2);
     const bool hubs = ctx->prm.hub_degree > 0 && !pruned;
     a.hubcutU = hubs ? (int32_t)std::min<int64_t>(cnt_ge(g.cntU_ge, ctx->prm.hub_degree), pU) : 0;
     a.hubcutV = hubs ? (int32_t)std::min<int64_t>(cnt_ge(g.cntV_ge, ctx->prm.hub_degree), pV) : 0;
@@ -767,7 +838,6 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     a.skip_zero = 1;
     a.fallen = (a.emit == 1 && P * 100 >= (int64_t)ctx->prm.emit_bitmap_min_pct * n) ? w.fallen : nullptr;
     a.sbits = a.emit == 2 ? w.fallen : nullptr;  // the gather's bitmap is free in a scatter
-    a.round0 = (ctx->prm.round0 && w.l0 && (a.searchU || a.searchV)) ? 1 : 0;
     a.l0 = w.l0;
     a.flags = w.flags;
     a.flag_first = 0;
@@ -792,15 +862,47 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     if (si.timed)
         for (int k = 0; k < 4; ++k)
             if (!w.ev[slot][k]) ABC_CU(cudaEventCreate(&w.ev[slot][k]));
+    if ((a.fallen != nullptr || a.sbits != nullptr) && w.fallen_dirty) {
+        ABC_CU(cudaMemsetAsync(w.fallen, 0, sizeof(uint32_t) * (size_t)((n + 31) / 32 + 1), ctx->stream));
+        w.fallen_dirty = false;
+    }
+    auto resident = [&](int &blocks_of, void (*k)(PeelArgs)) {
+        if (blocks_of <= 0) {
+            int per_sm = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, 0);
+            blocks_of = std::max(per_sm, 1) * ctx->num_sms;
+        }
+        return blocks_of;
+    };
+    if (Pu == 0 && !si.timed && ctx->prm.debug_stall_slots == 0) {
+        // every candidate is certain (a pruned query with equal bounds) or there is none: the masks are the prefixes,
+        // and no cascade is started (an empty one took 12 us)
+        a.ctl = nullptr;
+        a.fallen = nullptr;
+        if (a.emit == 1) {
+            k_gather<<<(unsigned)resident(ctx->gather_blocks, k_gather), 256, 0, ctx->stream>>>(a);
+            ctx->stats.launches++;
+        } else if (a.emit == 2) {
+            const int64_t gs = std::min<int64_t>((P + 2047) / 2048, (int64_t)ctx->num_sms * 8);
+            const int64_t ge = std::min<int64_t>(((n + 31) / 32 + 255) / 256, resident(ctx->expand_blocks, k_expand));
+            if (P > 0) k_scatter<<<(unsigned)gs, 256, 0, ctx->stream>>>(a);
+            ABC_CU(launch_k(ctx->prm.pdl != 0 && P > 0, k_expand, ge, 256, ctx->stream, (size_t)0, a));
+            ctx->stats.launches += P > 0 ? 2 : 1;
+        }
+        ABC_CU(cudaGetLastError());
+        w.ctl_host[slot] = PeelCtl{};
+        w.pending[slot] = true;
+        w.last = slot;
+        ctx->stats.mode = mode;
+        ctx->stats.grid_blocks = blocks;
+        ctx->pending_async = true;
+        return sync_and_check ? peel_finish(ctx) : ABCORE_OK;
+    }
     if (w.q_dirty) {
         ABC_CU(cudaMemsetAsync(w.q, 0xff, sizeof(unsigned long long) * (size_t)w.qcap, ctx->stream));
         w.q_dirty = false;
     }
     ABC_CU(cudaMemsetAsync(ctl, 0, sizeof(PeelCtl), ctx->stream));
-    if ((a.fallen != nullptr || a.sbits != nullptr) && w.fallen_dirty) {
-        ABC_CU(cudaMemsetAsync(w.fallen, 0, sizeof(uint32_t) * (size_t)((n + 31) / 32 + 1), ctx->stream));
-        w.fallen_dirty = false;
-    }
     if (t_init) ABC_CU(cudaEventRecord(w.ev[slot][0], ctx->stream));
     // the kernels after the count init follow it as programmatic dependents, except right after
     // a timing event (which must see the kernel before it end)
@@ -847,7 +949,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
             // the initial candidate violators' rows (their count is below the bound, so each row
             // is shorter than the bound)
             const int64_t gr = std::min<int64_t>((Pu + 255) / 256, (int64_t)ctx->num_sms * 16);
-            switch (ctx->prm.round0_variant) {
+            switch (round0_variant) {
                 case 1: ABC_CU(launch_k(pdl && prev_k, k_round0<4, 8>, gr, 256, ctx->stream, (size_t)0, a)); break;
                 case 2: ABC_CU(launch_k(pdl && prev_k, k_round0<16, 4>, gr, 256, ctx->stream, (size_t)0, a)); break;
                 case 3: ABC_CU(launch_k(pdl && prev_k, k_round0<8, 8>, gr, 256, ctx->stream, (size_t)0, a)); break;
@@ -875,12 +977,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
             const int64_t ns = a.round0 ? Pu
                                         : (a.searchU ? 0 : (int64_t)pU - a.hubcutU) + (a.searchV ? 0 : (int64_t)pV - a.hubcutV);
             // at most the blocks that fit at once: fewer blocks, fewer reservations on the queue
-            if (ctx->scan_blocks <= 0) {
-                int per_sm = 0;
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scan, 256, 0);
-                ctx->scan_blocks = std::max(per_sm, 1) * ctx->num_sms;
-            }
-            const int64_t gsc = std::min<int64_t>((ns + 255) / 256, ctx->scan_blocks);
+            const int64_t gsc = std::min<int64_t>((ns + 255) / 256, resident(ctx->scan_blocks, k_scan));
             ABC_CU(launch_k(pdl && prev_k, k_scan, gsc, 256, ctx->stream, (size_t)0, a));
             ctx->stats.launches++;
         }
@@ -896,21 +993,11 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     ABC_CU(launch_k(pdl && prev_k, k_cascade, blocks, 256, ctx->stream, (size_t)0, a));
     ctx->stats.launches++;
     if (a.emit == 1) {
-        if (ctx->gather_blocks <= 0) {
-            int per_sm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gather, 256, 0);
-            ctx->gather_blocks = std::max(per_sm, 1) * ctx->num_sms;
-        }
-        ABC_CU(launch_k(pdl, k_gather, ctx->gather_blocks, 256, ctx->stream, (size_t)0, a));
+        ABC_CU(launch_k(pdl, k_gather, resident(ctx->gather_blocks, k_gather), 256, ctx->stream, (size_t)0, a));
         ctx->stats.launches++;
     }
     if (a.emit == 2) {
-        if (ctx->expand_blocks <= 0) {
-            int per_sm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_expand, 256, 0);
-            ctx->expand_blocks = std::max(per_sm, 1) * ctx->num_sms;
-        }
-        const int64_t ge = std::min<int64_t>(((n + 31) / 32 + 255) / 256, ctx->expand_blocks);
+        const int64_t ge = std::min<int64_t>(((n + 31) / 32 + 255) / 256, resident(ctx->expand_blocks, k_expand));
         ABC_CU(launch_k(pdl, k_expand, ge, 256, ctx->stream, (size_t)0, a));
         ctx->stats.launches++;
     }
@@ -921,6 +1008,8 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     w.last = slot;
     ctx->stats.mode = mode;
     ctx->stats.grid_blocks = blocks;
+    ctx->log(1, "peel (%d,%d): %lld candidates, counting mode %d, first round about %.0f entries%s", alpha, beta, (long long)P, mode,
+             first_round_entries(g, alpha, beta), a.round0 ? ", walked first" : "");
     ctx->pending_async = true;
     if (sync_and_check) return peel_finish(ctx);
     return ABCORE_OK;

@@ -75,11 +75,11 @@ __device__ __forceinline__ bool cand_of(const PeelArgs &a, int32_t y, bool upper
 // neighbour falling), so no borrow crosses into the other half.
 // Slot of vertex x's count (PeelArgs::swz): the odd multiplier makes the per-layer map a
 // bijection of the layer's power-of-two range.
-constexpr unsigned long long SWZ_MUL = 0x9E3779B1ull;
+constexpr uint32_t SWZ_MUL = 0x9E3779B1u;
 __device__ __forceinline__ int64_t cnt_slot(const PeelArgs &a, int32_t x) {
     if (!a.swz) return x;
-    if (x < a.nU) return (int64_t)(((unsigned long long)(uint32_t)x * SWZ_MUL) & a.swz_mask_u);
-    return a.swz_base_v + (int64_t)(((unsigned long long)(uint32_t)(x - a.nU) * SWZ_MUL) & a.swz_mask_v);
+    if (x < a.nU) return (int64_t)(((uint32_t)x * SWZ_MUL) & a.swz_mask_u);
+    return a.swz_base_v + (int64_t)(((uint32_t)(x - a.nU) * SWZ_MUL) & a.swz_mask_v);
 }
 __device__ __forceinline__ int cnt_load(const PeelArgs &a, int32_t x) {
     const int64_t s = cnt_slot(a, x);
@@ -244,30 +244,34 @@ __device__ __forceinline__ int chunks_of(int len, int chunk) { return (len + chu
 // whose neighbours are drawn like everyone else's falls. From there it gallops outward in
 // doubling steps until the boundary is bracketed, then bisects. The result does not depend on
 // frac; a good guess settles most rows in one sector where bisection reads log2(length / 8).
-// `probes` counts the sectors read.
+// `probes` counts the sectors read. The eight entries of a sector come in two 16-byte loads, entries before the open range
+// standing as below the bound and entries past it as not (they may belong to other rows: adj is 32-byte
+// aligned and its allocation ends on a whole sector), so one comparison mask gives the boundary. The
+// count init is bound by instructions as much as by its reads: testing eight entries one by one
+// took it 64 us for (5,3) on 80M edges, now 57 (2.3M probes of 4.7M candidates; what is left is the rate of random sectors).
 __device__ __forceinline__ int row_prefix(const int32_t *__restrict__ adj, int64_t s, int64_t e, int32_t bound,
                                           float frac, unsigned long long &probes) {
-    const int32_t *row = adj + s;
     const int d = (int)(e - s);
     int lo = 0, hi = d;  // the boundary (first index holding an id >= bound, or d) is in [lo, hi]
     int p = (int)(frac * (float)d);
     p = p < 0 ? 0 : (p >= d ? d - 1 : p);
-    const int mis = (int)((reinterpret_cast<uintptr_t>(row) >> 2) & 7);  // entries past a sector start
+    const int mis = (int)(s & 7);  // entries past a sector start
+    const int4 *const sectors = reinterpret_cast<const int4 *>(adj + (s - mis));
     int dist = 8;
     int dir = 0;  // 0: first probe; +1 / -1: galloping right / left; 2: bracketed, bisecting
     while (lo < hi) {  // p is in [lo, hi): every pass shrinks the range
-        const int w = ((p + mis) & ~7) - mis;
+        const int sec = (p + mis) >> 3, w = (sec << 3) - mis;  // the sector's first entry is row entry w
+        const int4 q0 = __ldg(&sectors[2 * sec]), q1 = __ldg(&sectors[2 * sec + 1]);
         const int w0 = max(w, lo), w1 = min(w + 8, hi);
-        int below = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int i = w + k;
-            if (i >= w0 && i < w1) below += __ldg(&row[i]) < bound ? 1 : 0;
-        }
+        // bit i: entry w + i is below the bound (ids and the bound are below 2^31: the difference's sign)
+        auto bit = [&](int32_t y, int i) { return ((uint32_t)(y - bound) >> 31) << i; };
+        uint32_t m = bit(q0.x, 0) | bit(q0.y, 1) | bit(q0.z, 2) | bit(q0.w, 3) | bit(q1.x, 4) | bit(q1.y, 5) | bit(q1.z, 6) | bit(q1.w, 7);
+        m = (m | ((1u << (w0 - w)) - 1u)) & ((1u << (w1 - w)) - 1u);
+        const int at = w + __popc(m);  // entries [w0, at) are below, [at, w1) are not
         probes++;
-        if (below > 0 && below < w1 - w0) return w0 + below;
-        const int want = below == 0 ? -1 : 1;
-        if (below == 0) hi = w0;
+        if (at > w0 && at < w1) return at;
+        const int want = at == w0 ? -1 : 1;
+        if (want < 0) hi = w0;
         else lo = w1;
         if (lo >= hi) break;
         if (dir == 0 || dir == want) {
@@ -314,6 +318,7 @@ __device__ __forceinline__ void process_items(const PeelArgs &a, unsigned long l
         c = (int)(it & 0xffffffffu);
         if (a.fallen != nullptr && c == 0) o = __ldg(&a.new2old[x]);  // caller id, for the bitmap
         int rl = row_len_of(a, x);
+        const int live = cnt_load(a, x);  // (with the row's length and place: one round trip for the three)
         const long long s0 = __ldg(&a.off[x]);
         // a chain step with a narrower V prefix: a U row's candidates are its entries below it
         if (x < a.nU && a.pV < a.pV_rows && rl > 0) {
@@ -322,7 +327,7 @@ __device__ __forceinline__ void process_items(const PeelArgs &a, unsigned long l
         }
         // a count of 0 means every candidate neighbour has fallen and decremented this vertex
         // already: walking its row would only decrement fallen vertices, so the walk is skipped
-        if (rl > 0 && cnt_load(a, x) == 0) rl = 0;
+        if (live == 0) rl = 0;
         start = s0 + (long long)c * a.chunk;
         len = min(a.chunk, rl - c * a.chunk);
         if (len < 0) len = 0;
@@ -493,6 +498,8 @@ __device__ __forceinline__ int cascade_loop(const PeelArgs &a, WarpSmem &sm, Lan
         const int nwk = (int)(blockDim.x >> 5) - obs;
         const unsigned long long t = ld_relaxed(&a.ctl->tail);
         const unsigned long long h = ld_relaxed(&a.ctl->head);
+        // nothing queued when the cascade starts: only items queue items, so nothing will be
+        if (t == 0) s_k = -1;
         if (nwk > 0 && t > h && h < CLOSED) {
             const unsigned long long kk = (t - h) / (unsigned long long)grab_div;
             const int k = (int)(kk < 1 ? 1 : (kk > MAX_GRAB ? MAX_GRAB : kk));
@@ -511,6 +518,7 @@ __device__ __forceinline__ int cascade_loop(const PeelArgs &a, WarpSmem &sm, Lan
         }
     }
     __syncthreads();
+    if (s_k < 0) return ld_relaxed_i32(&a.ctl->err) != 0 ? 0 : 1;
     if (watcher && a.trace != nullptr) {
         // Diagnostics: the watcher takes no work; its lane 0 samples done, tail and head about
         // every microsecond (the first TRACE_SAMPLES samples are kept) until the queue drains,
@@ -803,6 +811,10 @@ __device__ __forceinline__ void init_range(const PeelArgs &a, PushBuf<CAP> &pb, 
                 }
             }
         } else {
+            bool any = false;
+#pragma unroll
+            for (int k = 0; k < INIT_ILP; ++k) any |= viol[k];
+            if (__ballot_sync(ABC_FULL, any) == 0) continue;
 #pragma unroll
             for (int k = 0; k < INIT_ILP; ++k)
                 push_add(a, pb, pc, viol[k], x[k] < 0 ? 0 : x[k], len[k] > 0 ? 1 : 0, ls);  // chunk 0
@@ -898,22 +910,25 @@ __device__ __forceinline__ void scan_range(const PeelArgs &a, PushBuf<CAP> &pb, 
                 c[k] = cnt_load(a, x[k]);
             }
         }
+        bool viol[SCAN_ILP], any = false;
 #pragma unroll
         for (int k = 0; k < SCAN_ILP; ++k) {
-            bool viol = false;
+            viol[k] = x[k] >= 0 && c[k] < (x[k] < a.nU ? a.thrU : a.thrV);
+            scanned += x[k] >= 0 ? 1 : 0;
+            any |= viol[k];
+        }
+        if (__ballot_sync(ABC_FULL, any) == 0) continue;
+#pragma unroll
+        for (int k = 0; k < SCAN_ILP; ++k) {
             int nch = 0;
-            if (x[k] >= 0) {
-                const int thr = x[k] < a.nU ? a.thrU : a.thrV;
-                // (a candidate the count init queued as known dead is not queued twice)
-                viol = c[k] < thr && !(a.dead_own && !chain_alive(a, x[k]));
-                if (viol) {
-                    const int pl = __ldcg(&a.plen[x[k]]);
-                    if (a.round0 && pl < thr) viol = false;  // an initial violator: round0 walked it
-                    else nch = pl > 0 ? 1 : 0;               // chunk 0 (see process_items)
-                }
-                scanned++;
+            // (a candidate the count init queued as known dead is not queued twice)
+            if (viol[k] && a.dead_own && !chain_alive(a, x[k])) viol[k] = false;
+            if (viol[k]) {
+                const int pl = __ldcg(&a.plen[x[k]]);
+                if (a.round0 && pl < (x[k] < a.nU ? a.thrU : a.thrV)) viol[k] = false;  // an initial violator: round0 walked it
+                else nch = pl > 0 ? 1 : 0;                                             // chunk 0 (see process_items)
             }
-            push_add(a, pb, pc, viol, x[k] < 0 ? 0 : x[k], nch, ls);
+            push_add(a, pb, pc, viol[k], x[k] < 0 ? 0 : x[k], nch, ls);
         }
     }
     if (BLOCK) push_flush_block(a, pb, pc);
