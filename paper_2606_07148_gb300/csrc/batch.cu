@@ -139,7 +139,11 @@ __global__ void __launch_bounds__(BATCH_THREADS, MINB) k_batch(BatchArgs B) {
     a.flag_first = cd.first_block;
     a.flag_count = G;
     a.epoch = 1;
-    const int grab_div = max(1, G * (BATCH_THREADS / 32) / 8);
+    // Grabs of an even share for half a chain's warps. With an eighth of them, a short queue is handed out in grabs
+    // that leave most warps without a row while a few walk eight each. An eighth -> half: 144 pairs over 10M edges
+    // 3.76 -> 2.69 ms, 64 pairs over 1M 1.07 -> 0.96, 256 pairs over 100M 17.9 -> 17.2, over 250M 39.6 -> 39.2; 16
+    // pairs over 40M are the same (1.77, 1.81), and so is a share for every warp (2.58, 0.97, 17.4, 39.6, 1.85).
+    const int grab_div = max(1, G * (BATCH_THREADS / 32) / 2);
 
     const int64_t t0 = (int64_t)r * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)G * blockDim.x;
