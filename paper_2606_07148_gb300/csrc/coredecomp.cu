@@ -8,7 +8,7 @@
 // network node and its relation to degree and coreness", 2016; asynchronous form: Sariyuce,
 // Seshadhri and Pinar, "Local algorithms for hierarchical dense subgraph discovery", 2018). A peel
 // goes through every k and every cascade level inside it, one after the other: on a 20M-edge power-law graph
-// 1,322 levels of a few vertices each, 15.9 ms of latency. The h-index rounds need 24 to 45 there and the
+// 1,322 levels of a few vertices each, 15.9 ms of latency. The h-index rounds need up to 60 there and the
 // work of about eight passes over the edges, most of it in the first, wide rounds: 3.1 ms, bound by
 // the latency of the later rounds' long rows and barriers.
 //
