@@ -310,10 +310,11 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "hub_degree"* [256] rows of at least this degree always count by search (0: none).
  *   "probe_bytes"* [32] the cost model's price of a search probe (steers search vs stream).
  *   "round0"* [by query] 1: walk the initial violators' rows with no-return decrements first; 0: queue
- *                       them. Until it is set, queries whose first round is long take 1 (with form 4).
- *   "round0_variant"* [0] that walk's form: 0..3 lane-per-entry (entries in flight / blocks an SM:
- *                       8/any, 4/8, 16/4, 8/8), 4 four rows per warp, 5 the same in one 1024-thread
- *                       block per SM summing hub decrements in shared memory.
+ *                       them. Until it is set, queries whose first round is long take 1.
+ *   "round0_variant"* [by query; 0 where "round0" is set and this is not] that walk's form: 0..3
+ *                       lane-per-entry (entries in flight / blocks an SM: 8/any, 4/8, 16/4, 8/8), 4
+ *                       four rows per warp, 5 the same in one 1024-thread block per SM summing hub
+ *                       decrements in shared memory. By query: 4, for the longest walks 5.
  *   "round0_hub"* [16384] hubs per layer in variant 5's table (0..28672).
  *   "count_swizzle" [1] counts in the per-layer multiplicative slot order (0: vertex order).
  *   "pdl" [1]           later kernels launch as programmatic dependents of the one before.

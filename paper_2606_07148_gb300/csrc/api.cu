@@ -607,7 +607,7 @@ int abcore_get_param(abcore_ctx *ctx, const char *name, int64_t *value) {
     else if (k == "flush_steps") *value = p.flush_steps;
     else if (k == "packed_counts") *value = p.packed_counts;
     else if (k == "round0") *value = p.round0 > 0 ? 1 : 0;
-    else if (k == "round0_variant") *value = p.round0_variant;
+    else if (k == "round0_variant") *value = std::max(p.round0_variant, 0);
     else if (k == "round0_hub") *value = p.round0_hub;
     else if (k == "count_swizzle") *value = p.count_swizzle;
     else if (k == "pdl") *value = p.pdl;

@@ -142,8 +142,9 @@ struct Params {
                                // no-return atomics when a layer counts by search (k_round0), instead
                                // of queueing them; -1, until it is set: where that saves enough
                                // (first_round_entries)
-    int round0_variant = 0;    // k_round0's compiled (entries per lane per step, blocks per SM) pair:
-                               // 0 (8, any), 1 (4, 8), 2 (16, 4), 3 (8, 8); 4: rows four at a time;
+    int round0_variant = -1;   // k_round0's compiled (entries per lane per step, blocks per SM) pair;
+                               // -1, until it is set: 4 or 5 by the length of the walk where round0
+                               // is -1 too, else 0. 0 (8, any), 1 (4, 8), 2 (16, 4), 3 (8, 8); 4: rows four at a time;
                                // 5: rows four at a time, hub decrements summed in shared memory
     int round0_hub = 16384;    // variant 5: hub counts per layer kept in each block's table
     int count_swizzle = 1;     // single peel: counts in the swizzled layout (see PeelArgs::swz); 0: in

@@ -47,6 +47,11 @@ constexpr int64_t SMALL_QUERY_VERTICES = 1 << 14, SMALL_QUERY_ENTRIES = 1 << 19;
 
 // First rounds of at least this many entries walk the initial violators' rows without returns (unless "round0" is set)
 constexpr double ROUND0_MIN_ENTRIES = 2e6;
+// ... and of at least this many with the hub table, unless the form is set: its start and its write-back are paid once,
+// and the longer the walk, the more decrements it absorbs. Whole queries, rows alone against the table: 22M entries
+// (300M edges, (30,100)) 360 / 406 us, 25M ((64,64)) 362 / 366, 46M (600M edges, (40,40), (64,64), (128,128)) 735 / 762,
+// 594 / 577, 564 / 569; 112M (1.5B edges, (64,64)) 1228 / 1143.
+constexpr double ROUND0_HUB_ENTRIES = 8e7;
 constexpr int SWIZZLE_MAX_PCT = 30;  // counts are spread when candidates are less than this share of the vertices
 
 constexpr int INIT_THREADS = 256;
@@ -805,7 +810,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     int round0 = ctx->prm.round0, round0_variant = ctx->prm.round0_variant;
     if (round0 < 0) {
         round0 = !pruned && mode == 3 && first_round_entries(g, alpha, beta) >= ROUND0_MIN_ENTRIES ? 1 : 0;
-        round0_variant = 4;
+        if (round0_variant < 0) round0_variant = first_round_entries(g, alpha, beta) >= ROUND0_HUB_ENTRIES ? 5 : 4;
     }
     if (round0 && (a.searchU || a.searchV) && w.l0_cap < Pu) {
         ctx->release(w.l0);

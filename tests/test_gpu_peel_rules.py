@@ -81,3 +81,20 @@ def test_long_first_rounds_are_walked():
         assert np.array_equal(mu.cpu().numpy(), wu) and np.array_equal(mv.cpu().numpy(), wv), (a, b)
         assert (core.stats()["round0_rows"] > 0) == (a > 2), (a, b)
     core.close()
+
+
+def test_a_chosen_form_is_used_where_the_rule_walks():
+    nU, nV, eu, ev = synth.make_graph("peel-4Mx2M-80M", device="cuda")
+    off, adj = oracle.build_csr(nU, nV, eu.cpu().numpy(), ev.cpu().numpy())
+    wu, wv, _ = oracle.peel_many(nU, nV, off, adj, [(50, 50)])[50, 50]
+    core = ABCore(0)
+    core.load_edges(nU, nV, eu, ev)
+    for variant in (None, 5, 0, 2):  # (None: by rule, rows without the hub table at this length)
+        if variant is not None:
+            core.set_param("round0_variant", variant)
+        core.set_param("reset_stats", 1)
+        mu, mv = core.compute(50, 50)
+        assert np.array_equal(mu.cpu().numpy(), wu) and np.array_equal(mv.cpu().numpy(), wv), variant
+        st = core.stats()
+        assert st["round0_rows"] > 0 and (st["hub_decrements"] > 0) == (variant == 5), variant
+    core.close()
