@@ -331,7 +331,8 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "batch_entries"* [1024] entries a warp walks per batch (128..2^24; the rest is re-queued).
  *   "batch_entries_small"* [512] the limit when a warp's grab leaves the queue nearly empty (0 off).
  *   "local_rounds" [256] batches a warp may chain on its own pushes (0..4096).
- *   "flush_steps"* [16]  steps a buffered push may wait before its warp flushes.
+ *   "flush_steps"* [16; 1 for single peels of large bounds] steps a buffered push may wait before its
+ *                       warp flushes.
  * Batch:
  *   "batch_wave"* [4, 8 or 16, by the size of the graph]  chains per wave (0..32; 0: all at once).
  *   "batch_plain_below"* [0] pairs with alpha below this run as single peels, not chains.

@@ -604,7 +604,7 @@ int abcore_get_param(abcore_ctx *ctx, const char *name, int64_t *value) {
     else if (k == "local_rounds") *value = p.local_rounds;
     else if (k == "batch_entries_small") *value = p.batch_entries_small;
     else if (k == "batch_entries") *value = p.batch_entries;
-    else if (k == "flush_steps") *value = p.flush_steps;
+    else if (k == "flush_steps") *value = p.flush_steps < 0 ? FLUSH_STEPS : p.flush_steps;
     else if (k == "packed_counts") *value = p.packed_counts;
     else if (k == "round0") *value = p.round0 > 0 ? 1 : 0;
     else if (k == "round0_variant") *value = std::max(p.round0_variant, 0);

@@ -700,7 +700,7 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
         // chains keep counts in vertex order: every step scans all of a chain's candidates in
         // order, which the swizzled layout would turn into random sector reads (measured slower)
         B.swz = 0;
-        B.flush_steps = ctx->prm.flush_steps;
+        B.flush_steps = ctx->prm.flush_steps < 0 ? FLUSH_STEPS : ctx->prm.flush_steps;
         B.qcap = b->qcap;
         B.timeout_ns = (unsigned long long)ctx->prm.timeout_ms * 1000000ull;
         B.prof = b->prof ? b->prof + wi * MAX_CHAINS_PER_WAVE * PROF_STRIDE : nullptr;

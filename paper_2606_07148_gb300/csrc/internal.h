@@ -136,7 +136,7 @@ struct Params {
     int chunk = 1024;
     int batch_entries = 1024;  // see PeelArgs (1024 kept a 94k-candidate, 18-level cascade 4.5x
                                // faster than 4096; the autotuner may raise it)
-    int flush_steps = 16;
+    int flush_steps = -1;      // -1, until it is set: by the query's bounds in a single peel (peel_compute), else 16
     int packed_counts = 1;     // batch chains keep 16-bit counts when every degree fits
     int round0 = -1;           // single peel: walk the initial candidate violators' rows with
                                // no-return atomics when a layer counts by search (k_round0), instead
@@ -206,6 +206,7 @@ struct Graph {
     int64_t n() const { return (int64_t)nU + nV; }
 };
 
+constexpr int FLUSH_STEPS = 16;         // "flush_steps" until it is set
 constexpr int ROUND0_HUB_MAX = 28672;  // "round0_hub": two layers' tables of ints in one block's shared memory
 
 constexpr int CTL_RING = 64;  // peels that may be in flight (ABCORE_ASYNC) before a forced wait

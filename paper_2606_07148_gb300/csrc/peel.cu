@@ -47,6 +47,15 @@ constexpr int64_t SMALL_QUERY_VERTICES = 1 << 14, SMALL_QUERY_ENTRIES = 1 << 19;
 
 // First rounds of at least this many entries walk the initial violators' rows without returns (unless "round0" is set)
 constexpr double ROUND0_MIN_ENTRIES = 2e6;
+// ... and no bound is above this: a walked row is shorter than its bound, and eight lanes take a long one as a chain of
+// steps while few rows are there to share. Queued / walked: 80M edges, (300,10) 411 / 462 us, (10,300) 331 / 389,
+// (112,386) 310 / 420, (500,500) 177 / 351; 300M edges, (250,30) 594 / 521, (200,200) 414 / 379, (112,386) 387 / 435.
+constexpr int ROUND0_MAX_BOUND = 256;
+// Queries whose bounds sum to more hand every push over at once and queue their first round, unless "flush_steps" and
+// "round0" are set: few vertices fall and each opens a long row. Pushes waiting one step (queued) / 16 steps (walked):
+// 80M edges, (112,386) 224 / 420 us, (250,250) 299 / 498, (500,500) 162 / 351, but (180,180) 225 / 251, (128,30) 318 /
+// 275, (20,160) 279 / 251; 300M edges, (500,500) 469 / 654, (112,386) 384 / 435, but (200,200) 428 / 379, (250,30) 639 / 521.
+constexpr int64_t LONG_BOUNDS = 400;
 // ... and of at least this many with the hub table, unless the form is set: its start and its write-back are paid once,
 // and the longer the walk, the more decrements it absorbs. Whole queries, rows alone against the table: 22M entries
 // (300M edges, (30,100)) 360 / 406 us, 25M ((64,64)) 362 / 366, 46M (600M edges, (40,40), (64,64), (128,128)) 735 / 762,
@@ -793,7 +802,8 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     a.thrV = beta;
     a.chunk = std::max(ctx->prm.chunk, 32);
     a.batch_entries = ctx->prm.batch_entries;
-    a.flush_steps = ctx->prm.flush_steps;
+    const bool long_bounds = (int64_t)alpha + beta > LONG_BOUNDS;
+    a.flush_steps = ctx->prm.flush_steps >= 0 ? ctx->prm.flush_steps : long_bounds ? 1 : FLUSH_STEPS;
     a.local_rounds = ctx->prm.local_rounds;
     a.batch_entries_small = ctx->prm.batch_entries_small;
     a.phases = ctx->prm.log_level >= 2 ? 1 : 0;
@@ -809,7 +819,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     // crossing is looked for in it, which runs half again as fast.
     int round0 = ctx->prm.round0, round0_variant = ctx->prm.round0_variant;
     if (round0 < 0) {
-        round0 = !pruned && mode == 3 && first_round_entries(g, alpha, beta) >= ROUND0_MIN_ENTRIES ? 1 : 0;
+        round0 = !pruned && mode == 3 && !long_bounds && std::max(alpha, beta) <= ROUND0_MAX_BOUND && first_round_entries(g, alpha, beta) >= ROUND0_MIN_ENTRIES ? 1 : 0;
         if (round0_variant < 0) round0_variant = first_round_entries(g, alpha, beta) >= ROUND0_HUB_ENTRIES ? 5 : 4;
     }
     if (round0 && (a.searchU || a.searchV) && w.l0_cap < Pu) {

@@ -98,3 +98,20 @@ def test_a_chosen_form_is_used_where_the_rule_walks():
         st = core.stats()
         assert st["round0_rows"] > 0 and (st["hub_decrements"] > 0) == (variant == 5), variant
     core.close()
+
+
+@pytest.mark.parametrize("pair", [(200, 200), (200, 201), (256, 20), (257, 20), (20, 257), (500, 500)])
+def test_large_bounds(pair):
+    # at and past the bounds from which first rounds are queued and pushes handed over at once
+    nU, nV = 20001, 10003
+    eu, ev = synth.chung_lu_edges(nU, nV, 3_000_000, 2.1, 2.2, 5, device="cuda")
+    off, adj = oracle.build_csr(nU, nV, eu.cpu().numpy(), ev.cpu().numpy())
+    wu, wv, _ = oracle.peel_many(nU, nV, off, adj, [pair])[pair]
+    core = ABCore(0)
+    core.load_edges(nU, nV, eu, ev)
+    for setting in ({}, {"round0": 1}, {"flush_steps": 16}):
+        for k, v in setting.items():
+            core.set_param(k, v)
+        mu, mv = core.compute(*pair)
+        assert np.array_equal(mu.cpu().numpy(), wu) and np.array_equal(mv.cpu().numpy(), wv), setting
+    core.close()
