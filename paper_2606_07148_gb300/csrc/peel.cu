@@ -55,6 +55,7 @@ constexpr int ROUND0_MAX_BOUND = 256;
 // "round0" are set: few vertices fall and each opens a long row. Pushes waiting one step (queued) / 16 steps (walked):
 // 80M edges, (112,386) 224 / 420 us, (250,250) 299 / 498, (500,500) 162 / 351, but (180,180) 225 / 251, (128,30) 318 /
 // 275, (20,160) 279 / 251; 300M edges, (500,500) 469 / 654, (112,386) 384 / 435, but (200,200) 428 / 379, (250,30) 639 / 521.
+constexpr int WIDE_BOUND = 128;  // see where the grab is chosen
 constexpr int64_t LONG_BOUNDS = 400;
 // ... and of at least this many with the hub table, unless the form is set: its start and its write-back are paid once,
 // and the longer the walk, the more decrements it absorbs. Whole queries, rows alone against the table: 22M entries
@@ -838,8 +839,11 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     // queue of 20,000 items, 31 each, and the tickets they held beyond it drew most later items to them
     // too (5M edges, (20,20) / (40,40): 152 / 218 us, with half the warps 71 / 81); after a long first round
     // what is queued is little and deep, and all warps share it.
+    // So do they with one large bound: its few rows are long (half / all warps: 10M edges, (10,300) 453 / 143 us, (300,10)
+    // 167 / 129, (180,180) 407 / 354; 80M edges, (10,300) 332 / 352, (300,10) 417 / 419, (180,180) 249 / 251).
     const int warps = blocks * (256 / 32);
-    a.grab_div = ctx->prm.grab_div > 0 ? ctx->prm.grab_div : std::max(1, a.round0 ? warps : warps / 2);
+    const bool wide = !long_bounds && std::max(alpha, beta) > WIDE_BOUND;
+    a.grab_div = ctx->prm.grab_div > 0 ? ctx->prm.grab_div : std::max(1, a.round0 || wide ? warps : warps / 2);
     const bool hubs = ctx->prm.hub_degree > 0 && !pruned;
     a.hubcutU = hubs ? (int32_t)std::min<int64_t>(cnt_ge(g.cntU_ge, ctx->prm.hub_degree), pU) : 0;
     a.hubcutV = hubs ? (int32_t)std::min<int64_t>(cnt_ge(g.cntV_ge, ctx->prm.hub_degree), pV) : 0;
