@@ -592,6 +592,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             leave = __shfl_sync(ABC_FULL, leave, 0);
             if (leave) break;
             upto = __shfl_sync(ABC_FULL, upto, 0);
+            __syncwarp();  // lane 0's acquire of the count comes before every lane's reads of the ring (a shuffle orders nothing)
             const int n = (int)(upto - k);
             Fetched f{};
             if (lane < n) {
@@ -643,6 +644,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             }
             const int n = (int)min(done - k, 32ull);
             __threadfence_block();
+            __syncwarp();  // (lane 0 has seen the count: every lane reads what it stands for after that)
             Answer a{};
             if (lane < n) a = answers[(k + lane) % SERVE_RING];
             __syncwarp();
@@ -709,6 +711,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
                 continue;
             }
             __threadfence_block();
+            __syncwarp();  // (lane 0 has seen the count: every lane reads the entry after that)
             const Fetched f = ring[k % SERVE_RING];
             Change ch{};
             const int st = apply_update<true>(S, f.op, f.x, f.y, f.px, f.py, ch);
