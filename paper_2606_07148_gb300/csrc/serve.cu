@@ -180,6 +180,14 @@ __device__ __forceinline__ int32_t ins_capacity(int32_t used) {
     return c;
 }
 
+// Sign of life of the warps that work on an update, in shared memory (null: nobody waits for them). One is given at
+// every vertex they take up and every BEAT_STEPS steps along a row, so whoever waits can tell a long update
+// from one that is stuck, however many levels and entries it has.
+constexpr int BEAT_STEPS = 256;
+__device__ __forceinline__ void beat_on(unsigned *beat) {
+    if (beat != nullptr && (threadIdx.x & 31) == 0) atomicAdd(beat, 1u);
+}
+
 // Visit the current neighbours of w: base row minus tombstones, plus live inserted neighbours.
 // Warp-collective: lanes stride the base row, then the inserted segment. Each lane hands f up to NB of them at once
 // (-1: none), so that what f reads of them is read together: what a re-peel waits for is round trips to L2, and
@@ -187,8 +195,10 @@ __device__ __forceinline__ int32_t ins_capacity(int32_t used) {
 // took six of them a step.
 constexpr int NB = 4;
 template <class F>
-__device__ __forceinline__ void for_neighbours(const ServeArgs &A, const TargetDev &S, int32_t w, F f) {
+__device__ __forceinline__ void for_neighbours(const ServeArgs &A, const TargetDev &S, int32_t w, unsigned *beat, F f) {
     const int lane = threadIdx.x & 31;
+    int step = 0;
+    beat_on(beat);
     const int64_t s = __ldg(&A.off[w]), e = __ldg(&A.off[w + 1]);
     const int2 seg = S.ins[w];
     int32_t z[NB];
@@ -204,18 +214,21 @@ __device__ __forceinline__ void for_neighbours(const ServeArgs &A, const TargetD
         for (int k = 0; k < NB; ++k)
             if (gone[k] & 1u) z[k] = -1;
         f(z);
+        if ((++step & (BEAT_STEPS - 1)) == 0) beat_on(beat);
     }
     for (int32_t i = lane; i - lane < seg.y; i += 32 * NB) {
 #pragma unroll
         for (int k = 0; k < NB; ++k) z[k] = i + 32 * k < seg.y ? S.pool[seg.x + i + 32 * k] : -1;
         f(z);
+        if ((++step & (BEAT_STEPS - 1)) == 0) beat_on(beat);
     }
 }
 
 // Warp-collective: position in the pool of `key` in segment seg, or -1.
-__device__ __forceinline__ int32_t ins_find(const TargetDev &S, int2 seg, int32_t key) {
+__device__ __forceinline__ int32_t ins_find(const TargetDev &S, int2 seg, int32_t key, unsigned *beat) {
     const int lane = threadIdx.x & 31;
     for (int32_t i0 = 0; i0 < seg.y; i0 += 32) {
+        if (i0 > 0 && (i0 & (32 * BEAT_STEPS - 1)) == 0) beat_on(beat);
         const unsigned m = __ballot_sync(ABC_FULL, i0 + lane < seg.y && S.pool[seg.x + i0 + lane] == key);  // live entries are distinct
         if (m) return seg.x + i0 + __ffs(m) - 1;
     }
@@ -230,11 +243,14 @@ __device__ __forceinline__ int32_t append_need(int2 seg) {
 }
 
 // Warp-collective: append y to x's inserted neighbours (segment seg), moving the segment to `at` where it needs room.
-__device__ __forceinline__ void ins_append(TargetDev &S, int32_t x, int2 seg, int32_t y, int32_t at) {
+__device__ __forceinline__ void ins_append(TargetDev &S, int32_t x, int2 seg, int32_t y, int32_t at, unsigned *beat) {
     const int lane = threadIdx.x & 31;
     const bool moves = append_need(seg) > 0;
     if (moves)
-        for (int32_t i = lane; i < seg.y; i += 32) S.pool[at + i] = S.pool[seg.x + i];
+        for (int32_t i = lane; i < seg.y; i += 32) {
+            S.pool[at + i] = S.pool[seg.x + i];
+            if (((i >> 5) & (BEAT_STEPS - 1)) == BEAT_STEPS - 1) beat_on(beat);
+        }
     if (lane == 0) {
         const int32_t to = moves ? at : seg.x;
         S.pool[to + seg.y] = y;
@@ -254,7 +270,7 @@ __device__ __forceinline__ void bq_push(BlockQueue &Q, int32_t z) { Q.q[atomicAd
 // Cascade inside the core after a delete: members whose in-core count fell below their bound
 // leave, lowering their member neighbours' counts (queued on the exact crossing). Vertices
 // leaving at cascade level L get certificate level base + L.
-__device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y) {
+__device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y, unsigned *beat) {
     __shared__ int tail;
     __shared__ int64_t base_s;
     BlockQueue Q{S.q, &tail};
@@ -274,7 +290,7 @@ __device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int3
         for (int i = head + warp; i < end; i += nwarps) {
             const int32_t w = S.q[i];
             if ((threadIdx.x & 31) == 0) S.rho[w] = base_s + level;
-            for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
+            for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
                 bool in[NB];
 #pragma unroll
                 for (int k = 0; k < NB; ++k) in[k] = z[k] >= 0 && S.M[z[k]];
@@ -300,7 +316,7 @@ __device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int3
 }
 
 // Region growth and peel after an insert with an endpoint outside the core (see the header).
-__device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y, int32_t ep) {
+__device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y, int32_t ep, unsigned *beat) {
     __shared__ int tail;
     __shared__ int64_t base_s;
     BlockQueue Q{S.q, &tail};
@@ -328,7 +344,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
         for (int i = head + warp; i < end; i += nwarps) {
             const int32_t w = S.q[i];
             const int64_t rw = S.rho[w];
-            for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
+            for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
                 bool in[NB];
                 int64_t rho[NB];
                 int32_t deg[NB];
@@ -352,7 +368,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
     for (int i = warp; i < R; i += nwarps) {
         const int32_t w = S.q[i];
         int c = 0;
-        for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
+        for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
 #pragma unroll
             for (int k = 0; k < NB; ++k) {
                 const int32_t y = max(z[k], 0);
@@ -384,7 +400,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
         for (int i = head + warp; i < end; i += nwarps) {
             const int32_t w = S.q[i];
             if (lane == 0) S.rho[w] = base_s + level;
-            for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
+            for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
                 bool in[NB];
 #pragma unroll
                 for (int k = 0; k < NB; ++k) in[k] = z[k] >= 0 && S.mark[z[k]] == ep;
@@ -404,7 +420,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
     for (int i = warp; i < R; i += nwarps) {
         const int32_t w = S.q[i];
         if (S.mark[w] != ep) continue;
-        for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
+        for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
 #pragma unroll
             for (int k = 0; k < NB; ++k) {
                 const int32_t y = max(z[k], 0);
@@ -445,7 +461,7 @@ constexpr int POOL_FULL = 1;
 // status, or POOL_FULL with the view unchanged (admission by memory: a new edge needs room in
 // both endpoints' pool segments). Warp-collective; CORE: the view has a core (M, cnt).
 template <bool CORE>
-__device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int32_t y, int64_t px, int64_t py, Change &ch) {
+__device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int32_t y, int64_t px, int64_t py, Change &ch, unsigned *beat) {
     const int lane = threadIdx.x & 31;
     // one round trip for all of it
     const bool base = px >= 0;
@@ -461,15 +477,15 @@ __device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int
         ch.cx = S.cnt[x];
         ch.cy = S.cnt[y];
     }
-    const int32_t qx = base ? -1 : ins_find(S, sx, y);
+    const int32_t qx = base ? -1 : ins_find(S, sx, y, beat);
     const bool present = base ? ((tw >> (px & 31)) & 1u) == 0 : qx >= 0;
     if (op == ABCORE_INSERT) {
         if (present) return ABCORE_EEXIST;
         if (!base) {
             const int32_t nx = append_need(sx), ny = append_need(sy);
             if ((int64_t)top + nx + ny > (int64_t)S.pool_cap) return POOL_FULL;
-            ins_append(S, x, sx, y, top);
-            ins_append(S, y, sy, x, top + nx);
+            ins_append(S, x, sx, y, top, beat);
+            ins_append(S, y, sy, x, top + nx, beat);
             if (lane == 0 && nx + ny > 0) *S.pool_top = top + nx + ny;
         }
         ch.dx++;
@@ -477,7 +493,7 @@ __device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int
     } else {
         if (!present) return ABCORE_ENOENT;
         if (!base) {
-            const int32_t qy = ins_find(S, sy, x);
+            const int32_t qy = ins_find(S, sy, x, beat);
             if (lane == 0) {
                 S.pool[qx] = -1;
                 S.pool[qy] = -1;
@@ -515,12 +531,18 @@ __device__ __forceinline__ unsigned long long ld_shared(const unsigned long long
 }
 
 // Limit of a wait of one of a block's warps on another: the other may itself be in its idle spell. Records
-// ABCORE_ETIMEDOUT and returns true once the wait that began with since = 0 has taken that long (the clock is
-// read only while waiting: it takes longer than a step of an update).
-__device__ __forceinline__ bool wait_over(const ServeArgs &A, unsigned long long &since) {
+// ABCORE_ETIMEDOUT and returns true once the wait that began with w = {} has taken that long without a sign of life of
+// the warps that work on an update: a re-peel may take longer than any limit, and is waited for while it gets on. (The
+// clock is read only while waiting: it takes longer than a step of an update.)
+struct Wait {
+    unsigned long long since = 0;
+    unsigned beat = 0;
+};
+__device__ __forceinline__ bool wait_over(const ServeArgs &A, Wait &w, const unsigned *beat) {
     const unsigned long long now = abc::now_ns();
-    if (since == 0) since = now;
-    if (now - since <= A.idle_ns + A.timeout_ns) return false;
+    const unsigned b = *(const volatile unsigned *)beat;
+    if (w.since == 0 || b != w.beat) w = Wait{now, b};
+    if (now - w.since <= A.idle_ns + A.timeout_ns) return false;
     abc::set_error(A.err, ABCORE_ETIMEDOUT);
     return true;
 }
@@ -538,12 +560,14 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
     __shared__ volatile int s_stop;     // the main warp has left: nothing follows s_done
     __shared__ int s_job;               // what the waiting warps are to help with: 0 nothing more, 1 a region, 2 a cascade
     __shared__ int32_t s_x, s_y, s_ep;
+    __shared__ unsigned s_beat;         // see beat_on
     TargetDev S = A.targets[blockIdx.x];
     const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long k0 = A.progress_dev[t];
     if (threadIdx.x == 0) {
         s_fetched = s_done = s_sent = k0;
         s_closed = s_stop = 0;
+        s_beat = 0;
     }
     __syncthreads();
     if (warp == work_warps()) {
@@ -553,7 +577,8 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             unsigned long long upto = k;  // requests [k, upto) are next
             int leave = 0;
             if (lane == 0) {
-                unsigned long long t0 = abc::now_ns();
+                const unsigned long long t0 = abc::now_ns();
+                Wait w;
                 unsigned sl = 32;
                 for (;;) {
                     if (s_stop || abc::ld_relaxed_i32(A.err)) {  // this target is held back, or the session failed
@@ -567,7 +592,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
                     }
                     const unsigned long long room = ld_shared(&s_done) + SERVE_RING - k;
                     if (room == 0) {  // the main warp is at work
-                        if (wait_over(A, t0)) {
+                        if (wait_over(A, w, &s_beat)) {
                             leave = 1;
                             break;
                         }
@@ -632,13 +657,14 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
         if (lane == 0) s_closed = 1;
     } else if (warp == work_warps() + 1) {
         // ---- respond ----
-        unsigned long long k = k0, since = 0;
+        unsigned long long k = k0;
+        Wait w;
         for (;;) {
             const int stop = s_stop;
             __threadfence_block();
             const unsigned long long done = __shfl_sync(ABC_FULL, ld_shared(&s_done), 0);
             if (k == done) {
-                if (__shfl_sync(ABC_FULL, stop || wait_over(A, since), 0)) break;
+                if (__shfl_sync(ABC_FULL, stop || wait_over(A, w, &s_beat), 0)) break;
                 __nanosleep(32);
                 continue;
             }
@@ -672,10 +698,11 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             __threadfence_system();
             __syncwarp();
             if (lane == 0) {
+                A.progress_dev[t] = k;  // (answered, not only applied: a loop that is launched again goes on here)
                 st_sys(&A.progress_host[t], k);
                 *(volatile unsigned long long *)&s_sent = k;
             }
-            since = 0;
+            w = Wait{};
         }
     } else if (warp > 0) {
         // ---- the main warp's helpers ----
@@ -684,12 +711,13 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             const int job = s_job;
             const int32_t x = s_x, y = s_y, ep = s_ep;
             if (job == 0) break;
-            if (job == 1) insert_region(A, S, x, y, ep);
-            else delete_cascade(A, S, x, y);
+            if (job == 1) insert_region(A, S, x, y, ep, &s_beat);
+            else delete_cascade(A, S, x, y, &s_beat);
         }
     } else {
         // ---- main ----
-        unsigned long long k = k0, since = 0;
+        unsigned long long k = k0;
+        Wait w;
         int32_t ep = *S.epoch;
         auto all_hands = [&](int job, int32_t x, int32_t y) {
             if (lane == 0) {
@@ -706,7 +734,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             __threadfence_block();
             const unsigned long long have = __shfl_sync(ABC_FULL, ld_shared(&s_fetched), 0);
             if (k == have) {
-                if (__shfl_sync(ABC_FULL, closed || wait_over(A, since), 0)) break;
+                if (__shfl_sync(ABC_FULL, closed || wait_over(A, w, &s_beat), 0)) break;
                 __nanosleep(20);
                 continue;
             }
@@ -714,7 +742,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             __syncwarp();  // (lane 0 has seen the count: every lane reads the entry after that)
             const Fetched f = ring[k % SERVE_RING];
             Change ch{};
-            const int st = apply_update<true>(S, f.op, f.x, f.y, f.px, f.py, ch);
+            const int st = apply_update<true>(S, f.op, f.x, f.y, f.px, f.py, ch, &s_beat);
             if (st == POOL_FULL) {
                 // hold request k back: the loop closes at k for every block, the host grows this
                 // target's pool and relaunches, and k is processed then (its answer is unchanged)
@@ -736,22 +764,22 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
                         }
                     } else {  // (a delete that takes an endpoint below its bound)
                         all_hands(2, f.x, f.y);
-                        delete_cascade(A, S, f.x, f.y);
+                        delete_cascade(A, S, f.x, f.y, &s_beat);
                         moved = true;
                     }
                 } else if (f.op == ABCORE_INSERT && ((!ch.mx && ch.dx >= tx) || (!ch.my && ch.dy >= ty))) {
                     ep += 2;
                     all_hands(1, f.x, f.y);
-                    insert_region(A, S, f.x, f.y, ep);
+                    insert_region(A, S, f.x, f.y, ep, &s_beat);
                     moved = true;
                 }
             }
             __syncwarp();
             const int bits = moved ? (S.M[f.x] ? 1 : 0) | (S.M[f.y] ? 2 : 0) : (ch.mx ? 1 : 0) | (ch.my ? 2 : 0);
-            since = 0;
+            w = Wait{};
             bool stuck = false;
             while (!stuck && k - __shfl_sync(ABC_FULL, ld_shared(&s_sent), 0) >= SERVE_RING) {  // the respond warp is behind
-                stuck = __shfl_sync(ABC_FULL, wait_over(A, since), 0);
+                stuck = __shfl_sync(ABC_FULL, wait_over(A, w, &s_beat), 0);
                 __nanosleep(64);
             }
             if (stuck) break;
@@ -768,7 +796,6 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
         if (lane == 0) {
             s_stop = 1;
             *S.epoch = ep;
-            A.progress_dev[t] = k;
         }
     }
 }
@@ -869,7 +896,7 @@ __global__ void __launch_bounds__(32) k_gfq_apply(ServeArgs A, TargetDev V, int 
     const int64_t px = warp_find(A.adj, __ldg(&A.off[x]), __ldg(&A.off[x + 1]), y);
     const int64_t py = px < 0 ? -1 : warp_find(A.adj, __ldg(&A.off[y]), __ldg(&A.off[y + 1]), x);
     Change ch{};
-    const int st = apply_update<false>(V, op, x, y, px, py, ch);
+    const int st = apply_update<false>(V, op, x, y, px, py, ch, nullptr);
     if (threadIdx.x == 0) {
         ids[0] = x;
         ids[1] = y;
@@ -940,7 +967,7 @@ __global__ void k_gfq_round(ServeArgs A, TargetDev V, int32_t alpha, int32_t bet
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = w0; i < nin; i += nw) {
         const int32_t w = fin[i];
-        for_neighbours(A, V, w, [&](const int32_t (&z)[NB]) {
+        for_neighbours(A, V, w, nullptr, [&](const int32_t (&z)[NB]) {
             bool in[NB];
 #pragma unroll
             for (int k = 0; k < NB; ++k) in[k] = z[k] >= 0 && alive[z[k]];
