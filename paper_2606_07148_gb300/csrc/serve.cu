@@ -558,6 +558,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
     __shared__ unsigned long long s_fetched, s_done, s_sent;
     __shared__ volatile int s_closed;   // the fetch warp has left: nothing follows s_fetched
     __shared__ volatile int s_stop;     // the main warp has left: nothing follows s_done
+    __shared__ volatile int s_failed;   // the session has failed: what was fetched is left alone
     __shared__ int s_job;               // what the waiting warps are to help with: 0 nothing more, 1 a region, 2 a cascade
     __shared__ int32_t s_x, s_y, s_ep;
     __shared__ unsigned s_beat;         // see beat_on
@@ -566,7 +567,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
     const unsigned long long k0 = A.progress_dev[t];
     if (threadIdx.x == 0) {
         s_fetched = s_done = s_sent = k0;
-        s_closed = s_stop = 0;
+        s_closed = s_stop = s_failed = 0;
         s_beat = 0;
     }
     __syncthreads();
@@ -581,7 +582,9 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
                 Wait w;
                 unsigned sl = 32;
                 for (;;) {
-                    if (s_stop || abc::ld_relaxed_i32(A.err)) {  // this target is held back, or the session failed
+                    const int err = abc::ld_relaxed_i32(A.err);
+                    if (s_stop || err) {  // this target is held back, or the session failed
+                        if (err) s_failed = 1;
                         leave = 1;
                         break;
                     }
@@ -593,6 +596,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
                     const unsigned long long room = ld_shared(&s_done) + SERVE_RING - k;
                     if (room == 0) {  // the main warp is at work
                         if (wait_over(A, w, &s_beat)) {
+                            s_failed = 1;
                             leave = 1;
                             break;
                         }
@@ -732,6 +736,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
         for (;;) {
             const int closed = s_closed;
             __threadfence_block();
+            if (__shfl_sync(ABC_FULL, s_failed, 0)) break;
             const unsigned long long have = __shfl_sync(ABC_FULL, ld_shared(&s_fetched), 0);
             if (k == have) {
                 if (__shfl_sync(ABC_FULL, closed || wait_over(A, w, &s_beat), 0)) break;
@@ -790,6 +795,7 @@ __global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A)
             }
             ++k;
             __syncwarp();
+            if (moved && __shfl_sync(ABC_FULL, abc::ld_relaxed_i32(A.err), 0)) break;  // (a re-peel ran out of levels)
         }
         all_hands(0, 0, 0);
         __threadfence_block();
