@@ -62,8 +62,11 @@ namespace {
 
 // Threads that work on an update; two more warps fetch and respond. A region's vertices are walked a warp each, so
 // the more the better (4 targets, 2,000 updates, regions of 25 vertices: 9.5, 9.2 and 8.4 ms with 256, 512 and
-// 960), while every target has an SM to itself; with more targets than SMs the small block lets several share one.
-constexpr int SERVE_WORK = 960, SERVE_WORK_SHARED = 256;
+// 960), while every target has an SM to itself. With more targets than SMs, blocks small enough that all of them run at
+// once: a target without a place waits until the others leave, after an idle spell. 400 updates, targets / SMs 160 / 152,
+// 300, 440, 600, 740: 0.70, 0.89, 1.10, 202, 202 ms with 256 (three blocks an SM), 0.73, 0.92, 1.11, 1.31, 1.58 with 192
+// (five an SM, 48 registers a thread).
+constexpr int SERVE_WORK = 960, SERVE_WORK_3 = 256, SERVE_WORK_5 = 192;
 constexpr int SERVE_EXTRA = 64;
 __device__ __forceinline__ int work_threads() { return (int)blockDim.x - SERVE_EXTRA; }
 __device__ __forceinline__ int work_warps() { return work_threads() >> 5; }
@@ -551,7 +554,8 @@ __device__ __forceinline__ void st_sys_relaxed(unsigned long long *p, unsigned l
     asm volatile("st.relaxed.sys.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__global__ void __launch_bounds__(SERVE_WORK + SERVE_EXTRA) k_serve(ServeArgs A) {
+template <int WORK, int MINB>
+__global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A) {
     __shared__ Fetched ring[SERVE_RING];
     __shared__ Answer answers[SERVE_RING];
     // requests fetched, applied (and answered into the ring) and responded to; all only grow
@@ -1073,8 +1077,9 @@ static int launch_loop(abcore_ctx *ctx, ServeState *s) {
     A.timeout_ns = (unsigned long long)ctx->prm.timeout_ms * 1000000ull;
     cudaGetLastError();
     ABC_CU(cudaMemsetAsync(s->d_exit_at, 0xff, sizeof(unsigned long long), s->stream));
-    const int work = A.ntargets <= ctx->num_sms ? SERVE_WORK : SERVE_WORK_SHARED;
-    k_serve<<<A.ntargets, work + SERVE_EXTRA, 0, s->stream>>>(A);
+    if (A.ntargets <= ctx->num_sms) k_serve<SERVE_WORK, 1><<<A.ntargets, SERVE_WORK + SERVE_EXTRA, 0, s->stream>>>(A);
+    else if (A.ntargets <= 3 * ctx->num_sms) k_serve<SERVE_WORK_3, 3><<<A.ntargets, SERVE_WORK_3 + SERVE_EXTRA, 0, s->stream>>>(A);
+    else k_serve<SERVE_WORK_5, 5><<<A.ntargets, SERVE_WORK_5 + SERVE_EXTRA, 0, s->stream>>>(A);
     ABC_CU(cudaGetLastError());
     ABC_CU(cudaEventRecord(s->loop_done, s->stream));
     s->loop_launched = true;
