@@ -304,8 +304,10 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "algo" [0]          0 auto, 1 GCC (plain peel, Algorithm 1), 2 GCC+ (pruned by core numbers,
  *                       Algorithm 2; needs abcore_core_numbers first); auto takes GCC+ when it leaves
  *                       fewer vertices than GCC.
- *   "small_peel" [1]    a query with few candidates on a small graph runs whole in one block, a batch
- *                       of such queries a block per pair; 0: always the general peel.
+ *   "small_peel" [1]    a query on a small graph runs whole in one block, a batch of such queries a block
+ *                       per pair, unless a parameter of the kernels this replaces (single peel and
+ *                       cascade; for a batch "mode", "hub_degree", "probe_bytes", cascade and batch) has
+ *                       another value than its default; 0: always those kernels.
  *   "mode" [-1]         per-layer count init: -1 cost model, 0..3 bit 0 U by row search, bit 1 V.
  *   "hub_degree"* [256] rows of at least this degree always count by search (0: none).
  *   "probe_bytes"* [32] the cost model's price of a search probe (steers search vs stream).

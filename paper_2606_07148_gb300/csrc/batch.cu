@@ -608,13 +608,13 @@ static bool batch_packed(const abcore_ctx *ctx) {
 // narrow steps, until their counts no longer find room in L2. 16 chains of 6M vertices (12 MB of counts each), 256
 // pairs on 100M edges: waves of 2 / 4 / 8 / 16 34.9 / 25.0 / 21.1 / 19.6 ms; 0.6M vertices, 144 pairs on 10M edges: 9.9 / 6.4 /
 // 5.5 / 4.2; 30M vertices (60 MB each, 500M edges): 4 was the best.
-int batch_wave_of(const abcore_ctx *ctx) {
-    if (ctx->prm.batch_wave >= 0) return ctx->prm.batch_wave;
+static int wave_by_size(const abcore_ctx *ctx) {
     const int64_t bytes = (batch_packed(ctx) ? 2 : 4) * ctx->g.n();
     int w = 16;
     while (w > 4 && w * bytes > BATCH_WAVE_BYTES) w /= 2;
     return w;
 }
+int batch_wave_of(const abcore_ctx *ctx) { return ctx->prm.batch_wave >= 0 ? ctx->prm.batch_wave : wave_by_size(ctx); }
 
 // Chain workspaces: counts, queue, control block and barrier per concurrent chain, plus lvl.
 static int ensure_memory(abcore_ctx *ctx, BatchState *b, int want_chains) {
@@ -743,10 +743,12 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
 // start and end each, about 25 us whatever their size). 8 x 8 pairs: 3,500 vertices and 20k edges 84 us against 957
 // in chains; 15,010 and 200k 115 against 1,109; 35,000 and 800k 182 against 1,119; 21,000 and 1M 134 against 810.
 constexpr int64_t SMALL_BATCH_EDGES = 1 << 20;
+// ... and nothing is asked for that only chains have (a parameter of theirs, timed kernels, the timeline).
 static bool small_batch(const abcore_ctx *ctx) {
-    const Params &p = ctx->prm;
+    const Params &p = ctx->prm, d;
     return p.small_peel && ctx->g.n() <= abc::SMALL_MAX && ctx->g.m <= SMALL_BATCH_EDGES && p.timing == 0 && p.log_level < 2 &&
-           p.batch_plain_below == 0 && p.batch_seed == 0;
+           !kernels_steered(p) && p.batch_plain_below == d.batch_plain_below && p.batch_seed == d.batch_seed &&
+           p.packed_counts == d.packed_counts && (p.batch_wave < 0 || p.batch_wave == wave_by_size(ctx));
 }
 
 static int batch_small(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t *alphas, const int32_t *betas, uint8_t *d_masks_u,

@@ -191,6 +191,21 @@ struct Params {
                                // atomics on one address serialise (0 = off)
 };
 
+// Whether a parameter that steers the general peel's kernels, or those of single peels and batch chains alike, has been
+// set to something else: a query then takes them, however small its graph.
+inline bool kernels_steered(const Params &p) {
+    const Params d;
+    return p.chunk != d.chunk || p.batch_entries != d.batch_entries || p.flush_steps != d.flush_steps ||
+           p.blocks_per_sm != d.blocks_per_sm || p.mode != d.mode || p.hub_degree != d.hub_degree || p.probe_bytes != d.probe_bytes;
+}
+inline bool peel_steered(const Params &p) {
+    const Params d;
+    return kernels_steered(p) || p.grab_div != d.grab_div || p.local_rounds != d.local_rounds ||
+           p.batch_entries_small != d.batch_entries_small || p.round0 != d.round0 || p.round0_variant != d.round0_variant ||
+           p.round0_hub != d.round0_hub || p.count_swizzle != d.count_swizzle || p.pdl != d.pdl ||
+           p.emit_scatter_max_pct != d.emit_scatter_max_pct || p.emit_bitmap_min_pct != d.emit_bitmap_min_pct;
+}
+
 struct Graph {
     bool loaded = false;
     int32_t nU = 0, nV = 0;

@@ -719,11 +719,11 @@ static_assert(SMALL_QUERY_VERTICES <= abc::SMALL_MAX, "every candidate has its p
 
 // Whether a query runs in one block: one SM gets through the candidates and their rows in less than the
 // time the general peel's launches and levels take, and nothing that only the general peel has is asked
-// for (a set counting mode or first round, timed kernels, the queue trace, the stall hook).
+// for (a parameter of its kernels, timed kernels, the queue trace, the stall hook).
 static bool small_query(const abcore_ctx *ctx, int64_t entries, const uint8_t *mu, const uint8_t *mv) {
     const Params &p = ctx->prm;
     return p.small_peel && entries <= SMALL_QUERY_ENTRIES && ctx->g.n() <= SMALL_QUERY_VERTICES &&
-           p.mode < 0 && p.round0 <= 0 && p.timing == 0 && p.log_level < 2 && p.debug_stall_slots == 0 &&
+           !peel_steered(p) && p.timing == 0 && p.log_level < 2 && p.debug_stall_slots == 0 &&
            (mu != nullptr || ctx->g.nU == 0) && (mv != nullptr || ctx->g.nV == 0);
 }
 
