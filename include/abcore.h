@@ -311,12 +311,12 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "mode" [-1]         per-layer count init: -1 cost model, 0..3 bit 0 U by row search, bit 1 V.
  *   "hub_degree"* [256] rows of at least this degree always count by search (0: none).
  *   "probe_bytes"* [32] the cost model's price of a search probe (steers search vs stream).
- *   "round0"* [by query] 1: walk the initial violators' rows with no-return decrements first; 0: queue
- *                       them. Until it is set, queries whose first round is long take 1.
- *   "round0_variant"* [by query; 0 where "round0" is set and this is not] that walk's form: 0..3
- *                       lane-per-entry (entries in flight / blocks an SM: 8/any, 4/8, 16/4, 8/8), 4
- *                       four rows per warp, 5 the same in one 1024-thread block per SM summing hub
- *                       decrements in shared memory. By query: 4, for the longest walks 5.
+ *   "round0"* [-1]      1: walk the initial violators' rows with no-return decrements first; 0: queue
+ *                       them; -1: by query (long first rounds of short rows are walked).
+ *   "round0_variant"* [-1] that walk's form: 0..3 lane-per-entry (entries in flight / blocks an SM:
+ *                       8/any, 4/8, 16/4, 8/8), 4 four rows per warp, 5 the same in one 1024-thread
+ *                       block per SM summing hub decrements in shared memory; -1: by query (4, for the
+ *                       longest walks 5; 0 where "round0" is 1).
  *   "round0_hub"* [16384] hubs per layer in variant 5's table (0..28672).
  *   "count_swizzle" [1] counts in the per-layer multiplicative slot order (0: vertex order).
  *   "pdl" [1]           later kernels launch as programmatic dependents of the one before.
@@ -333,10 +333,11 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "batch_entries"* [1024] entries a warp walks per batch (128..2^24; the rest is re-queued).
  *   "batch_entries_small"* [512] the limit when a warp's grab leaves the queue nearly empty (0 off).
  *   "local_rounds" [256] batches a warp may chain on its own pushes (0..4096).
- *   "flush_steps"* [16; 1 for single peels of large bounds] steps a buffered push may wait before its
- *                       warp flushes.
+ *   "flush_steps"* [-1] steps a buffered push may wait before its warp flushes (1..2^20); -1: by query
+ *                       (16, for single peels of large bounds 1).
  * Batch:
- *   "batch_wave"* [4, 8 or 16, by the size of the graph]  chains per wave (0..32; 0: all at once).
+ *   "batch_wave"* [-1]  chains per wave (0..32; 0: all at once); -1: 4, 8 or 16 by the graph's size, and
+ *                       read as that number.
  *   "batch_plain_below"* [0] pairs with alpha below this run as single peels, not chains.
  *   "batch_seed"* [0]   1: seed each chain from the finished chain of the next smaller alpha.
  *   "packed_counts" [1] chains keep 16-bit counts whenever every degree fits.

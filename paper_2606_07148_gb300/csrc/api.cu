@@ -487,7 +487,7 @@ int abcore_set_param(abcore_ctx *ctx, const char *name, int64_t value) {
         p.count_swizzle = (int)value;
         free_batch(ctx);
     } else if (k == "round0_variant") {
-        if (value < 0 || value > 5) return ctx->fail(ABCORE_EINVAL, "round0_variant must be 0..5");
+        if (value < -1 || value > 5) return ctx->fail(ABCORE_EINVAL, "round0_variant must be -1 (by query) or 0..5");
         ABC_TRY(abcore_sync(ctx));
         p.round0_variant = (int)value;
     } else if (k == "round0_hub") {
@@ -499,11 +499,12 @@ int abcore_set_param(abcore_ctx *ctx, const char *name, int64_t value) {
         ABC_TRY(abcore_sync(ctx));
         p.pdl = (int)value;
     } else if (k == "round0") {
-        if (value < 0 || value > 1) return ctx->fail(ABCORE_EINVAL, "round0 must be 0 or 1");
+        if (value < -1 || value > 1) return ctx->fail(ABCORE_EINVAL, "round0 must be -1 (by query), 0 or 1");
         ABC_TRY(abcore_sync(ctx));
         p.round0 = (int)value;
     } else if (k == "flush_steps") {
-        if (value < 1 || value > (1 << 20)) return ctx->fail(ABCORE_EINVAL, "flush_steps must be in [1, 2^20]");
+        if (value != -1 && (value < 1 || value > (1 << 20)))
+            return ctx->fail(ABCORE_EINVAL, "flush_steps must be -1 (by query) or in [1, 2^20]");
         ABC_TRY(abcore_sync(ctx));
         p.flush_steps = (int)value;
         free_batch(ctx);
@@ -540,7 +541,7 @@ int abcore_set_param(abcore_ctx *ctx, const char *name, int64_t value) {
         if (value < 1) return ctx->fail(ABCORE_EINVAL, "probe_bytes must be >= 1");
         p.probe_bytes = (double)value;
     } else if (k == "batch_wave") {
-        if (value < 0 || value > 32) return ctx->fail(ABCORE_EINVAL, "batch_wave must be 0..32");
+        if (value < -1 || value > 32) return ctx->fail(ABCORE_EINVAL, "batch_wave must be -1 (by the graph's size) or 0..32");
         p.batch_wave = (int)value;
         free_batch(ctx);
     } else if (k == "batch_plain_below") {
@@ -604,10 +605,10 @@ int abcore_get_param(abcore_ctx *ctx, const char *name, int64_t *value) {
     else if (k == "local_rounds") *value = p.local_rounds;
     else if (k == "batch_entries_small") *value = p.batch_entries_small;
     else if (k == "batch_entries") *value = p.batch_entries;
-    else if (k == "flush_steps") *value = p.flush_steps < 0 ? FLUSH_STEPS : p.flush_steps;
+    else if (k == "flush_steps") *value = p.flush_steps;
     else if (k == "packed_counts") *value = p.packed_counts;
-    else if (k == "round0") *value = p.round0 > 0 ? 1 : 0;
-    else if (k == "round0_variant") *value = std::max(p.round0_variant, 0);
+    else if (k == "round0") *value = p.round0;
+    else if (k == "round0_variant") *value = p.round0_variant;
     else if (k == "round0_hub") *value = p.round0_hub;
     else if (k == "count_swizzle") *value = p.count_swizzle;
     else if (k == "pdl") *value = p.pdl;

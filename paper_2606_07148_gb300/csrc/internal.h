@@ -136,14 +136,14 @@ struct Params {
     int chunk = 1024;
     int batch_entries = 1024;  // see PeelArgs (1024 kept a 94k-candidate, 18-level cascade 4.5x
                                // faster than 4096; the autotuner may raise it)
-    int flush_steps = -1;      // -1, until it is set: by the query's bounds in a single peel (peel_compute), else 16
+    int flush_steps = -1;      // -1: by the query's bounds in a single peel (peel_compute), else 16
     int packed_counts = 1;     // batch chains keep 16-bit counts when every degree fits
     int round0 = -1;           // single peel: walk the initial candidate violators' rows with
                                // no-return atomics when a layer counts by search (k_round0), instead
-                               // of queueing them; -1, until it is set: where that saves enough
+                               // of queueing them; -1: where that saves enough
                                // (first_round_entries)
     int round0_variant = -1;   // k_round0's compiled (entries per lane per step, blocks per SM) pair;
-                               // -1, until it is set: 4 or 5 by the length of the walk where round0
+                               // -1: 4 or 5 by the length of the walk where round0
                                // is -1 too, else 0. 0 (8, any), 1 (4, 8), 2 (16, 4), 3 (8, 8); 4: rows four at a time;
                                // 5: rows four at a time, hub decrements summed in shared memory
     int round0_hub = 16384;    // variant 5: hub counts per layer kept in each block's table
@@ -169,8 +169,8 @@ struct Params {
     int batch_seed = 0;        // 1: a batch chain is seeded from the finished chain of the next
                                // smaller alpha with the same betas (its non-members are queued at
                                // once); measured no faster on the power-law grids, so off by default
-    int batch_wave = -1;       // chains sharing the GPU at once (0 = as many as fit, up to 32; -1, until it is
-                               // set: by the size of their counts, batch_wave_of)
+    int batch_wave = -1;       // chains sharing the GPU at once (0 = as many as fit, up to 32; -1: by the size
+                               // of their counts, batch_wave_of)
     int debug_stall_slots = 0; // test hook: queue slots reserved but never written
     int timing = 0;            // 1: CUDA events around each launch, summed into stats.kernel_ms
     int timing_kinds = 0xff;   // single peel: the kernel kinds (bit ABCORE_K_*) timed. An event
@@ -221,7 +221,7 @@ struct Graph {
     int64_t n() const { return (int64_t)nU + nV; }
 };
 
-constexpr int FLUSH_STEPS = 16;         // "flush_steps" until it is set
+constexpr int FLUSH_STEPS = 16;         // "flush_steps" where neither it nor the bounds say otherwise
 constexpr int ROUND0_HUB_MAX = 28672;  // "round0_hub": two layers' tables of ints in one block's shared memory
 
 constexpr int CTL_RING = 64;  // peels that may be in flight (ABCORE_ASYNC) before a forced wait

@@ -120,7 +120,7 @@ int autotune(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32_t *b
         for (const Knob &k : knobs) {
             int64_t cur = 0;
             abcore_get_param(ctx, k.name, &cur);
-            const Params before = ctx->prm;  // (a parameter that was never set follows its rule)
+            const Params before = ctx->prm;  // ("batch_wave" reads as what its rule gives, and goes on following it)
             int64_t keep = cur;
             for (int64_t v : k.values) {
                 if (v == cur) continue;
