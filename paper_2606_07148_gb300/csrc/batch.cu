@@ -231,6 +231,10 @@ __global__ void __launch_bounds__(abc::SMALL_THREADS, 1) k_batch_small(abc::Smal
     if (threadIdx.x == 0) host[p] = st;
 }
 
+// Pairs one launch of k_batch_emit writes at most (it holds them in shared memory; 16 chains have 4,080 distinct ones)
+constexpr int EMIT_PAIRS = 4096;
+static_assert(sizeof(int32_t) * (4 * MAX_CHAINS_PER_WAVE + 1 + 2 * EMIT_PAIRS) <= 48 * 1024, "a launch needs no larger limit");
+
 struct PairRef {
     int32_t chain;  // index into the wave's chains
     int32_t step;
@@ -716,19 +720,16 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
         cfg.numAttrs = 1;
         ABC_CU(cudaLaunchKernelExC(&cfg, (const void *)batch_kernel(ctx), args));
         ctx->stats.launches++;
-        if (!w.pairs.empty()) {
-            const int np = (int)w.pairs.size();
+        for (size_t p0 = 0; p0 < w.pairs.size(); p0 += EMIT_PAIRS) {
+            const int np = (int)std::min<size_t>(EMIT_PAIRS, w.pairs.size() - p0);
             const size_t shm = sizeof(int32_t) * (4 * cw + 1 + 2 * np);
-            if (shm > 200 * 1024) return ctx->fail(ABCORE_EINVAL, "too many pairs in one batch wave");
             // a wave whose chains have the columns 0, 1, ... of rows of at most 16
             const int words = !b->lvl_global && b->lvl_stride <= 16 ? b->lvl_stride / 4 : 0;
             auto *emit = words == 1 ? k_batch_emit<1> : words == 2 ? k_batch_emit<2> : words == 3 ? k_batch_emit<3>
                        : words == 4 ? k_batch_emit<4> : k_batch_emit<0>;
-            if (shm > 48 * 1024)
-                ABC_CU(cudaFuncSetAttribute(emit, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
             const int eg = (int)std::min<int64_t>((n + 255) / 256, (int64_t)ctx->num_sms * 8);
             emit<<<std::max(eg, 1), 256, shm, ctx->stream>>>(g.old2new, g.nU, g.nV, b->lvl, b->lvl_stride,
-                                                                     w.d_chains, cw, w.d_pairs, w.d_pidx, np, b->d_out);
+                                                                     w.d_chains, cw, w.d_pairs + p0, w.d_pidx + p0, np, b->d_out);
             ctx->stats.launches++;
         }
         for (int c = 0; c < cw; ++c)
@@ -866,7 +867,7 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
     }
     if (b->exec) {
         ABC_CU(cudaGraphLaunch(b->exec, ctx->stream));
-        for (auto &w : b->waves) ctx->stats.launches += 1 + (w.pairs.empty() ? 0 : 1);
+        for (auto &w : b->waves) ctx->stats.launches += 1 + (int64_t)((w.pairs.size() + EMIT_PAIRS - 1) / EMIT_PAIRS);
     } else {
         ABC_TRY(enqueue_batch(ctx, b));
     }

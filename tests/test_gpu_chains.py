@@ -95,3 +95,23 @@ def test_a_captured_plan_serves_any_buffers(small):
         for k, (wu, wv) in enumerate(want):
             assert np.array_equal(mu[k].cpu().numpy(), wu) and np.array_equal(mv[k].cpu().numpy(), wv), (shift, pairs[k])
     core.close()
+
+
+def test_more_pairs_than_one_launch_writes(small):
+    # many pairs given again and again: a wave's masks take several launches
+    nU, nV, eu, ev, off, adj = small
+    core = ABCore(0)
+    core.load_edges(nU, nV, eu.cuda(), ev.cuda())
+    core.set_param("small_peel", 0)
+    distinct = [(a, b) for a in range(1, 17) for b in (1, 2, 3, 5, 8, 13)]
+    rng = np.random.default_rng(3)
+    at = np.concatenate([rng.integers(0, len(distinct), 30_000), np.arange(len(distinct))])
+    want = [oracle.peel(nU, nV, off, adj, *p) for p in distinct]
+    wu, wv = (torch.from_numpy(np.stack([w[k] for w in want])).cuda() for k in (0, 1))
+    for shift in (0, 1):
+        mu = torch.full((len(at) * nU + shift,), 7, dtype=torch.uint8, device="cuda")[shift:].view(len(at), nU)
+        mv = torch.full((len(at) * nV + shift,), 7, dtype=torch.uint8, device="cuda")[shift:].view(len(at), nV)
+        core.compute_batch([distinct[k][0] for k in at], [distinct[k][1] for k in at], mu, mv)
+        idx = torch.from_numpy(at).cuda()
+        assert torch.equal(mu, wu[idx]) and torch.equal(mv, wv[idx])
+    core.close()
