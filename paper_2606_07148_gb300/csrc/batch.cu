@@ -222,12 +222,13 @@ out:
 }
 
 // A batch of a small graph: one block per pair (small_peel.cuh). What each did goes to the host.
+template <bool LONG>
 __global__ void __launch_bounds__(abc::SMALL_THREADS, 1) k_batch_small(abc::SmallGraph G, const abc::SmallQuery *__restrict__ queries,
                                                                        uint8_t *masks_u, uint8_t *masks_v, abc::SmallStats *host) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ abc::SmallStats st;
     const int p = blockIdx.x;
-    abc::small_peel(G, queries[p], smem, masks_u + (size_t)p * G.nU, masks_v + (size_t)p * G.nV, &st);
+    abc::small_peel<LONG>(G, queries[p], smem, masks_u + (size_t)p * G.nU, masks_v + (size_t)p * G.nV, &st);
     if (threadIdx.x == 0) host[p] = st;
 }
 
@@ -745,8 +746,15 @@ static int enqueue_batch(abcore_ctx *ctx, BatchState *b) {
 // in chains; 15,010 and 200k 115 against 1,109; 35,000 and 800k 182 against 1,119; 21,000 and 1M 134 against 810.
 constexpr int64_t SMALL_BATCH_EDGES = 1 << 20;
 // ... and nothing is asked for that only chains have (a parameter of theirs, timed kernels, the timeline).
-static bool small_batch(const abcore_ctx *ctx) {
+// Few pairs of very many rows to walk at once are left to the chains too: 4 pairs with 33,000 rows of 30 entries each
+// 408 us a block per pair, 190 in chains.
+constexpr double SMALL_BATCH_ROWS = 16384;
+constexpr int32_t SMALL_BATCH_PAIRS = 32;
+static bool small_batch(const abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32_t *betas) {
     const Params &p = ctx->prm, d;
+    if (n < SMALL_BATCH_PAIRS && ctx->g.n() > SMALL_BATCH_ROWS)
+        for (int32_t i = 0; i < n; ++i)
+            if (first_round_rows(ctx->g, alphas[i], betas[i]) > SMALL_BATCH_ROWS) return false;
     return p.small_peel && ctx->g.n() <= abc::SMALL_MAX && ctx->g.m <= SMALL_BATCH_EDGES && p.timing == 0 && p.log_level < 2 &&
            !kernels_steered(p) && p.batch_plain_below == d.batch_plain_below && p.batch_seed == d.batch_seed &&
            p.packed_counts == d.packed_counts && (p.batch_wave < 0 || p.batch_wave == wave_by_size(ctx));
@@ -773,9 +781,10 @@ static int batch_small(abcore_ctx *ctx, BatchState *b, int32_t n, const int32_t 
     }
     const size_t smem = abc::small_smem(most);
     // (the largest: the limit belongs to the function, which other contexts launch too)
-    ABC_CU(cudaFuncSetAttribute(k_batch_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)abc::small_smem(abc::SMALL_MAX)));
+    auto *k = std::max(g.maxdegU, g.maxdegV) > abc::SMALL_LONG ? k_batch_small<true> : k_batch_small<false>;
+    ABC_CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)abc::small_smem(abc::SMALL_MAX)));
     ABC_CU(cudaMemcpyAsync(b->d_queries, b->h_queries, sizeof(abc::SmallQuery) * n, cudaMemcpyHostToDevice, ctx->stream));
-    k_batch_small<<<n, abc::SMALL_THREADS, smem, ctx->stream>>>({g.off, g.adj, g.old2new, g.nU, g.nV}, b->d_queries, d_masks_u, d_masks_v,
+    k<<<n, abc::SMALL_THREADS, smem, ctx->stream>>>({g.off, g.adj, g.old2new, g.nU, g.nV}, b->d_queries, d_masks_u, d_masks_v,
                                                                 b->h_small);
     ABC_CU(cudaGetLastError());
     ABC_CU(cudaStreamSynchronize(ctx->stream));
@@ -801,7 +810,7 @@ int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32
     const Graph &g = ctx->g;
     if (!ctx->batch) ctx->batch = new BatchState();
     BatchState *b = ctx->batch;
-    if (small_batch(ctx)) return batch_small(ctx, b, n, alphas, betas, d_masks_u, d_masks_v);
+    if (small_batch(ctx, n, alphas, betas)) return batch_small(ctx, b, n, alphas, betas, d_masks_u, d_masks_v);
     if (!b->d_out) ABC_TRY(ctx->alloc(&b->d_out, 2, "batch mask addresses"));
     if (!b->h_out) ABC_TRY(ctx->host_alloc(&b->h_out, 2, "batch mask addresses"));
     const bool same = b->exec && b->key_graph_n == g.n() &&

@@ -501,6 +501,7 @@ int cascade_grid(abcore_ctx *ctx);
 int batch_compute(abcore_ctx *ctx, int32_t n, const int32_t *alphas, const int32_t *betas,
                   uint8_t *d_masks_u, uint8_t *d_masks_v, bool sync_and_check);
 void free_batch(abcore_ctx *ctx);
+double first_round_rows(const Graph &g, int32_t alpha, int32_t beta);  // (peel.cu) expected initial violators
 int batch_wave_of(const abcore_ctx *ctx);  // "batch_wave", or what the loaded graph's size makes it
 
 // serve.cu

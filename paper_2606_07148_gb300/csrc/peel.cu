@@ -44,6 +44,9 @@ using abc::WarpSmem;
 // against 46 / 80 / 36; 15,010 and 200k 34 / 51 / 52 against 46 / 67 / 67; 30,000 and 400k 48 / 71 / 100 against
 // 46 / 55 / 164; 21,000 and 1M 46 / 46 / 95 against 33 / 46 / 83.
 constexpr int64_t SMALL_QUERY_VERTICES = 1 << 14, SMALL_QUERY_ENTRIES = 1 << 19;
+// ... and rows the first round is expected to have: 128 of them at a time take one SM about 0.7 us. (All of 16,000 rows of
+// 16 entries at once: 127 us in one block, 60 in the general peel.)
+constexpr double SMALL_QUERY_ROWS = 8192;
 
 // First rounds of at least this many entries walk the initial violators' rows without returns (unless "round0" is set)
 constexpr double ROUND0_MIN_ENTRIES = 2e6;
@@ -511,11 +514,12 @@ __global__ void __launch_bounds__(256) k_expand(PeelArgs a) {
 
 // The whole query in one block (small_peel.cuh). Its control block goes straight to the host's readback copy:
 // this kernel has no bounded wait that could fail.
+template <bool LONG>
 __global__ void __launch_bounds__(abc::SMALL_THREADS, 1) k_small(abc::SmallGraph G, abc::SmallQuery Q, uint8_t *mask_u, uint8_t *mask_v,
                                                                  PeelCtl *host) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ abc::SmallStats st;
-    abc::small_peel(G, Q, smem, mask_u, mask_v, &st);
+    abc::small_peel<LONG>(G, Q, smem, mask_u, mask_v, &st);
     if (threadIdx.x < 12) {
         const int k = threadIdx.x;
         host->st[k] = k == ST_INIT ? st.inits : k == ST_PROBES ? st.probes : k == ST_ENTRIES ? st.entries : k == ST_DECS ? st.decs
@@ -699,6 +703,18 @@ static double first_round_entries(const Graph &g, int32_t alpha, int32_t beta) {
     return layer(alpha, g.edgesU_ge, eV / m) + layer(beta, g.edgesV_ge, eU / m);
 }
 
+// Rows that round is expected to have: candidates whose expected count, to the nearest whole number, misses the bound.
+double first_round_rows(const Graph &g, int32_t alpha, int32_t beta) {
+    const double m = (double)std::max<int64_t>(g.m, 1);
+    auto layer = [&](int32_t thr, const std::vector<int64_t> &cnt, double f) {
+        if (thr <= 0) return 0.0;
+        const double top = f > 0.0 ? std::min((double)INT32_MAX, std::ceil(((double)thr - 0.5) / f)) : (double)INT32_MAX;
+        return (double)(cnt_ge(cnt, thr) - cnt_ge(cnt, (int32_t)top));
+    };
+    const double eU = (double)cnt_ge(g.edgesU_ge, alpha), eV = (double)cnt_ge(g.edgesV_ge, beta);
+    return layer(alpha, g.cntU_ge, eV / m) + layer(beta, g.cntV_ge, eU / m);
+}
+
 // With core numbers prepared, is the pruned peel (GCC+) the cheaper one? GCC+ initialises and
 // peels the vertices with core in [min(alpha, beta), max(alpha, beta)); the plain peel those
 // meeting their bound on full degree. Each side's vertex count stands for its cost: equal
@@ -720,9 +736,11 @@ static_assert(SMALL_QUERY_VERTICES <= abc::SMALL_MAX, "every candidate has its p
 // Whether a query runs in one block: one SM gets through the candidates and their rows in less than the
 // time the general peel's launches and levels take, and nothing that only the general peel has is asked
 // for (a parameter of its kernels, timed kernels, the queue trace, the stall hook).
-static bool small_query(const abcore_ctx *ctx, int64_t entries, const uint8_t *mu, const uint8_t *mv) {
+static bool small_query(const abcore_ctx *ctx, int32_t alpha, int32_t beta, const uint8_t *mu, const uint8_t *mv) {
     const Params &p = ctx->prm;
-    return p.small_peel && entries <= SMALL_QUERY_ENTRIES && ctx->g.n() <= SMALL_QUERY_VERTICES &&
+    return p.small_peel && ctx->g.n() <= SMALL_QUERY_VERTICES &&
+           cnt_ge(ctx->g.edgesU_ge, alpha) + cnt_ge(ctx->g.edgesV_ge, beta) <= SMALL_QUERY_ENTRIES &&
+           first_round_rows(ctx->g, alpha, beta) <= SMALL_QUERY_ROWS &&
            !peel_steered(p) && p.timing == 0 && p.log_level < 2 && p.debug_stall_slots == 0 &&
            (mu != nullptr || ctx->g.nU == 0) && (mv != nullptr || ctx->g.nV == 0);
 }
@@ -744,7 +762,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     const int32_t cU = pruned ? (int32_t)cnt_ge(ctx->pr.coreU_ge, dq) : 0;
     const int32_t cV = pruned ? (int32_t)cnt_ge(ctx->pr.coreV_ge, dq) : 0;
     const int64_t P = (int64_t)pU + pV, Pu = (int64_t)(pU - cU) + (pV - cV);
-    if (small_query(ctx, cnt_ge(ctx->g.edgesU_ge, alpha) + cnt_ge(ctx->g.edgesV_ge, beta), d_mask_u, d_mask_v)) {
+    if (small_query(ctx, alpha, beta, d_mask_u, d_mask_v)) {
         const int slot = w.next;
         if (w.pending[slot]) ABC_TRY(peel_finish(ctx));
         w.next = (w.next + 1) % CTL_RING;
@@ -758,12 +776,14 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
         const size_t smem = abc::small_smem(Pu);
         // (always the largest: the limit belongs to the function, which other contexts launch too)
         if (!ctx->small_allowed) {
-            ABC_CU(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)abc::small_smem(abc::SMALL_MAX)));
+            for (auto *f : {k_small<false>, k_small<true>})
+                ABC_CU(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)abc::small_smem(SMALL_QUERY_VERTICES)));
             ctx->small_allowed = true;
         }
         const abc::SmallGraph G{g.off, g.adj, g.old2new, nU, nV};
         const abc::SmallQuery Q{alpha, beta, pU, pV, cU, cV};
-        k_small<<<1, abc::SMALL_THREADS, smem, ctx->stream>>>(G, Q, d_mask_u, d_mask_v, w.ctl_host + slot);
+        auto *k = std::max(g.maxdegU, g.maxdegV) > abc::SMALL_LONG ? k_small<true> : k_small<false>;
+        k<<<1, abc::SMALL_THREADS, smem, ctx->stream>>>(G, Q, d_mask_u, d_mask_v, w.ctl_host + slot);
         ABC_CU(cudaGetLastError());
         ctx->stats.launches++;
         ctx->stats.mode = 3;
