@@ -173,11 +173,27 @@ __device__ __forceinline__ void core_rows(const CoreArgs &C, int32_t x, CoreBuf 
         if (r < nr) core_mark(C, b, nb, drops && v[r] > lo, y[r], next, count);
 }
 
-// A long row by the whole block.
+// How many of the ascending entries adj[s, f) are below `bound`: every thread probes a place, which cuts the row in 257.
+// Block-collective.
+__device__ __forceinline__ int row_end(const CoreArgs &C, int64_t s, int64_t f, int32_t bound) {
+    const int t = threadIdx.x;
+    int64_t a = s, b = f;  // entries before a are below, those from b on are not
+    while (b - a > CORE_THREADS) {
+        const int64_t len = b - a;
+        const int k = __syncthreads_count(__ldg(&C.adj[a + len * (t + 1) / (CORE_THREADS + 1)]) < bound);
+        if (k < CORE_THREADS) b = a + len * (k + 1) / (CORE_THREADS + 1);
+        if (k > 0) a = a + len * k / (CORE_THREADS + 1) + 1;
+    }
+    return (int)(a - s) + __syncthreads_count(a + t < b && __ldg(&C.adj[a + t]) < bound);
+}
+
+// A long row by the whole block: up to three passes over the entries that can count, none with a barrier in it. The new
+// value is searched for in the values kept in shared memory, or, with more than fit, in counts of them by value
+// (a search that read such rows again for every step took k_core 310 ms of 361 with 20 rows of 2M entries).
 __device__ __forceinline__ void core_long(const CoreArgs &C, int32_t x, int32_t *cache, CoreBuf &b, int &nb, int32_t *next, unsigned *count) {
     __shared__ int s_n[2];
-    __shared__ int64_t s_end;
-    const int t = threadIdx.x;
+    __shared__ int s_best, s_w[CORE_WARPS];
+    const int t = threadIdx.x, lane = t & 31;
     if (t == 0) {
         atomicExch(&C.queued[x], 0);
         __threadfence();
@@ -188,28 +204,22 @@ __device__ __forceinline__ void core_long(const CoreArgs &C, int32_t x, int32_t 
     const int64_t s = __ldg(&C.off[x]), f = __ldg(&C.off[x + 1]);
     const int e = ld_val(&C.val[x]);
     constexpr int LILP = 4;
-    // entries before the first id at or past `bound`; calls fn(index, id, value) on them
-    auto walk = [&](int32_t bound, auto fn) {
-        for (int64_t p0 = s; p0 < f; p0 += CORE_THREADS * LILP) {
+    // fn(index, value) on the row's first n entries
+    auto walk = [&](int n, auto fn) {
+        for (int i0 = t; i0 < n; i0 += CORE_THREADS * LILP) {
             int32_t y[LILP], v[LILP];
-            bool past = false;
 #pragma unroll
-            for (int q = 0; q < LILP; ++q) {
-                const int64_t p = p0 + q * CORE_THREADS + t;
-                y[q] = p < f ? __ldg(&C.adj[p]) : INT32_MAX;
-                past |= y[q] >= bound;
-            }
+            for (int q = 0; q < LILP; ++q) y[q] = i0 + q * CORE_THREADS < n ? __ldg(&C.adj[s + i0 + q * CORE_THREADS]) : -1;
 #pragma unroll
-            for (int q = 0; q < LILP; ++q) v[q] = y[q] < bound ? ld_val(&C.val[y[q]]) : -1;
+            for (int q = 0; q < LILP; ++q) v[q] = y[q] >= 0 ? ld_val(&C.val[y[q]]) : -1;
 #pragma unroll
             for (int q = 0; q < LILP; ++q)
-                if (y[q] < bound) fn((int)(p0 - s) + q * CORE_THREADS + t, y[q], v[q]);
-            if (__syncthreads_or(past)) break;
+                if (y[q] >= 0) fn(i0 + q * CORE_THREADS, v[q]);
         }
     };
     auto total = [&](int mine, int slot) {
         mine = __reduce_add_sync(ABC_FULL, mine);
-        if ((t & 31) == 0 && mine) atomicAdd(&s_n[slot], mine);
+        if (lane == 0 && mine) atomicAdd(&s_n[slot], mine);
         __syncthreads();
         const int r = s_n[slot];
         if (t == 0) s_n[slot ^ 1] = 0;
@@ -217,42 +227,84 @@ __device__ __forceinline__ void core_long(const CoreArgs &C, int32_t x, int32_t 
         return r;
     };
     int mine = 0;
-    walk(id_bound(C, upper, e), [&](int, int32_t, int32_t v) { mine += v >= e ? 1 : 0; });
+    walk(row_end(C, s, f, id_bound(C, upper, e)), [&](int, int32_t v) { mine += v >= e ? 1 : 0; });
     const int c = total(mine, 0);
     if (c >= e) return;
-    // the new value lies in [c, e): keep the values of the entries that can count for it
-    const int32_t bound = id_bound(C, upper, max(c, 1));
-    if (t == 0) s_end = 0;
-    __syncthreads();
-    int last = 0;
-    walk(bound, [&](int i, int32_t, int32_t v) {
-        if (i < CORE_CACHE) cache[i] = v;
-        last = i + 1;
-    });
-    last = __reduce_max_sync(ABC_FULL, last);
-    if ((t & 31) == 0) atomicMax((long long *)&s_end, (long long)last);
-    __syncthreads();
-    const int n = (int)s_end;
-    auto value = [&](int i) { return i < CORE_CACHE ? cache[i] : ld_val(&C.val[__ldg(&C.adj[s + i])]); };
-    int lo = c, hi = e - 1, slot = 1;
+    // the new value lies in [c, e), and the first n entries can count for it
+    const int n = row_end(C, s, f, id_bound(C, upper, max(c, 1)));
+    const bool kept = n <= CORE_CACHE;
+    int lo = c, hi = e - 1;
+    if (kept) {
+        walk(n, [&](int i, int32_t v) { cache[i] = v; });
+        __syncthreads();
+        int slot = 1;
+        while (lo < hi) {
+            const int mid = lo + ((hi - lo + 1) >> 1);
+            int k = 0;
+            for (int i = t; i < n; i += CORE_THREADS) k += cache[i] >= mid ? 1 : 0;
+            k = total(k, slot);
+            slot ^= 1;
+            if (k >= mid) lo = mid;
+            else hi = mid - 1;
+        }
+    }
+    // values from lo up, counted in steps of w: the last step k of which lo + k w entries reach that value holds the new one
     while (lo < hi) {
-        const int mid = lo + ((hi - lo + 1) >> 1);
-        int k = 0;
-        for (int i = t; i < n; i += CORE_THREADS) k += value(i) >= mid ? 1 : 0;
-        k = total(k, slot);
-        slot ^= 1;
-        if (k >= mid) lo = mid;
-        else hi = mid - 1;
+        const int w = (hi - lo + CORE_CACHE) / CORE_CACHE, bins = (hi - lo) / w + 1;
+        for (int i = t; i < bins; i += CORE_THREADS) cache[i] = 0;
+        if (t == 0) s_best = 0;
+        __syncthreads();
+        int top = 0;
+        walk(n, [&](int, int32_t v) {
+            if (v >= hi) ++top;
+            else if (v >= lo) atomicAdd(&cache[(v - lo) / w], 1);
+        });
+        top = __reduce_add_sync(ABC_FULL, top);
+        if (lane == 0 && top) atomicAdd(&cache[bins - 1], top);
+        __syncthreads();
+        // thread t: steps [b0, b1), after them those of the threads past it
+        const int per = (bins + CORE_THREADS - 1) / CORE_THREADS, b0 = min(t * per, bins), b1 = min(b0 + per, bins);
+        int sum = 0;
+        for (int k = b0; k < b1; ++k) sum += cache[k];
+        int run = sum;  // this lane's and the lanes' past it
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_down_sync(ABC_FULL, run, d);
+            if (lane + d < 32) run += o;
+        }
+        if (lane == 0) s_w[t >> 5] = run;
+        __syncthreads();
+        for (int k = (t >> 5) + 1; k < CORE_WARPS; ++k) run += s_w[k];
+        run -= sum;
+        for (int k = b1 - 1; k >= b0; --k) {
+            run += cache[k];
+            if (run >= lo + k * w) {
+                atomicMax(&s_best, k);
+                break;
+            }
+        }
+        __syncthreads();
+        lo += s_best * w;
+        hi = min(hi, lo + w - 1);
+        __syncthreads();
     }
     if (t == 0) {
         C.val[x] = lo;
         __threadfence();
     }
     __syncthreads();
-    for (int i0 = 0; i0 < n; i0 += CORE_THREADS) {
-        const int i = i0 + t;
-        const bool in = i < n && value(i) > lo;
-        core_mark(C, b, nb, in, in ? __ldg(&C.adj[s + i]) : 0, next, count);
+    for (int i0 = 0; i0 < n; i0 += CORE_THREADS * LILP) {
+        int32_t y[LILP];
+        bool in[LILP];
+#pragma unroll
+        for (int q = 0; q < LILP; ++q) {
+            const int i = i0 + q * CORE_THREADS + t;
+            y[q] = i < n ? __ldg(&C.adj[s + i]) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < LILP; ++q) in[q] = y[q] >= 0 && (kept ? cache[i0 + q * CORE_THREADS + t] : ld_val(&C.val[y[q]])) > lo;
+#pragma unroll
+        for (int q = 0; q < LILP; ++q) core_mark(C, b, nb, in[q], max(y[q], 0), next, count);
     }
     __syncthreads();
 }
