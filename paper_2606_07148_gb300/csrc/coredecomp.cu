@@ -32,24 +32,28 @@ namespace {
 
 constexpr int CORE_THREADS = 256;
 constexpr int CORE_WARPS = CORE_THREADS / 32;
-// rows by length: up to CORE_SMALL entries by eight lanes, up to CORE_MID by a warp (in registers), longer by a block
-constexpr int CORE_SMALL = 64, CORE_MID = 512;
+// rows by length: up to CORE_SMALL entries by eight lanes, up to CORE_MID by a warp (in registers), up to CORE_LONG by a
+// block, longer by the whole grid
+constexpr int CORE_SMALL = 64, CORE_MID = 512, CORE_LONG = 32768;
+constexpr int CLASSES = 4;        // 0: the longest
 constexpr int CORE_CACHE = 4096;  // values of a long row a block keeps in shared memory
 constexpr int CORE_BUF = 128;     // vertices a warp collects before it adds them to a list
+constexpr int HUGE_BATCH = 256;   // rows of class 0 the grid takes together
+constexpr int HUGE_CHUNK = 4096;  // entries of one a block takes at a time
 
 struct CoreArgs {
     const int64_t *off;
     const int32_t *adj;
     int32_t nU, nV;
-    int32_t hU[2], hV[2];           // vertices of each layer with more than CORE_MID / CORE_SMALL edges, and
-    int32_t zU, zV;                 // with any (prefixes)
+    int32_t hU[CLASSES], hV[CLASSES];  // vertices of each layer in the classes up to this one (prefixes; the last: all with an edge)
     const int32_t *gU, *gV;         // vertices of each layer with at least t edges, t = 0 .. maxdeg + 1
     int32_t maxdeg;
     int32_t *val;                   // [n] values, by internal id: in the end the core numbers
     int32_t *queued;                // [n] 1: in the list of this or the next round, not yet looked at
-    int32_t *list[2];               // [n] vertices to look at, by class: long rows from 0, middle ones from the
-                                    // number of long ones, short ones after those
-    unsigned *count;                // [3][3] list lengths: [round % 3][class]
+    int32_t *list[2];               // [n] vertices to look at, each class from the number of vertices in those before it
+    unsigned *count;                // [3][CLASSES] list lengths: [round % 3][class]
+    int32_t *hcnt, *hval, *hist;    // [HUGE_BATCH] of a batch of class 0: entries at or above the value, the new value or -1;
+                                    // [HUGE_BATCH][CORE_CACHE] entries by value
     PeelCtl *ctl;
     unsigned *bar;
     unsigned long long timeout_ns;
@@ -70,13 +74,14 @@ __device__ __forceinline__ int32_t id_bound(const CoreArgs &C, bool upper, int32
 __device__ __forceinline__ int row_class(const CoreArgs &C, int32_t x) {
     const bool upper = x < C.nU;
     const int32_t i = upper ? x : x - C.nU;
-    return i < (upper ? C.hU[0] : C.hV[0]) ? 0 : i < (upper ? C.hU[1] : C.hV[1]) ? 1 : 2;
+    int c = 0;
+#pragma unroll
+    for (int k = 0; k < CLASSES - 1; ++k) c += i >= (upper ? C.hU[k] : C.hV[k]) ? 1 : 0;
+    return c;
 }
 
 // Where a class's part of a list starts.
-__device__ __forceinline__ int64_t list_start(const CoreArgs &C, int cls) {
-    return cls == 0 ? 0 : cls == 1 ? (int64_t)C.hU[0] + C.hV[0] : (int64_t)C.hU[1] + C.hV[1];
-}
+__device__ __forceinline__ int64_t list_start(const CoreArgs &C, int cls) { return cls == 0 ? 0 : (int64_t)C.hU[cls - 1] + C.hV[cls - 1]; }
 
 // Per warp: vertices to look at next round, collected before they take places in the lists.
 struct CoreBuf {
@@ -88,9 +93,9 @@ __device__ __forceinline__ void core_flush(const CoreArgs &C, CoreBuf &b, int &n
     __syncwarp();
     for (int i0 = 0; i0 < nb; i0 += 32) {
         const int32_t x = i0 + lane < nb ? b.x[i0 + lane] : -1;
-        const int cls = x >= 0 ? row_class(C, x) : 3;
+        const int cls = x >= 0 ? row_class(C, x) : CLASSES;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < CLASSES; ++c) {
             const unsigned m = __ballot_sync(ABC_FULL, cls == c);
             if (m == 0) continue;
             unsigned base = 0;
@@ -187,6 +192,40 @@ __device__ __forceinline__ int row_end(const CoreArgs &C, int64_t s, int64_t f, 
     return (int)(a - s) + __syncthreads_count(a + t < b && __ldg(&C.adj[a + t]) < bound);
 }
 
+// Entries at or above each value, from counts of them by value: bins[k] (k < n) counts values lo + k w to lo + k w + w - 1, the last
+// bin all above too. Returns the last k of which at least lo + k w entries lie in bins k and up (0 if none).
+// Block-collective; ends with a barrier, s_w: a word a warp.
+template <class F>
+__device__ __forceinline__ int last_reached(F bin, int n, int lo, int w, int *s_best, int *s_w) {
+    const int t = threadIdx.x, lane = t & 31;
+    if (t == 0) *s_best = 0;
+    // thread t: bins [b0, b1), above them those of the threads past it
+    const int per = (n + CORE_THREADS - 1) / CORE_THREADS, b0 = min(t * per, n), b1 = min(b0 + per, n);
+    int sum = 0;
+    for (int k = b0; k < b1; ++k) sum += bin(k);
+    int run = sum;  // this lane's and those of the lanes past it
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_down_sync(ABC_FULL, run, d);
+        if (lane + d < 32) run += o;
+    }
+    if (lane == 0) s_w[t >> 5] = run;
+    __syncthreads();
+    for (int k = (t >> 5) + 1; k < CORE_WARPS; ++k) run += s_w[k];
+    run -= sum;
+    for (int k = b1 - 1; k >= b0; --k) {
+        run += bin(k);
+        if (run >= lo + k * w) {
+            atomicMax(s_best, k);
+            break;
+        }
+    }
+    __syncthreads();
+    const int best = *s_best;
+    __syncthreads();
+    return best;
+}
+
 // A long row by the whole block: up to three passes over the entries that can count, none with a barrier in it. The new
 // value is searched for in the values kept in shared memory, or, with more than fit, in counts of them by value
 // (a search that read such rows again for every step took k_core 310 ms of 361 with 20 rows of 2M entries).
@@ -252,7 +291,6 @@ __device__ __forceinline__ void core_long(const CoreArgs &C, int32_t x, int32_t 
     while (lo < hi) {
         const int w = (hi - lo + CORE_CACHE) / CORE_CACHE, bins = (hi - lo) / w + 1;
         for (int i = t; i < bins; i += CORE_THREADS) cache[i] = 0;
-        if (t == 0) s_best = 0;
         __syncthreads();
         int top = 0;
         walk(n, [&](int, int32_t v) {
@@ -262,31 +300,8 @@ __device__ __forceinline__ void core_long(const CoreArgs &C, int32_t x, int32_t 
         top = __reduce_add_sync(ABC_FULL, top);
         if (lane == 0 && top) atomicAdd(&cache[bins - 1], top);
         __syncthreads();
-        // thread t: steps [b0, b1), after them those of the threads past it
-        const int per = (bins + CORE_THREADS - 1) / CORE_THREADS, b0 = min(t * per, bins), b1 = min(b0 + per, bins);
-        int sum = 0;
-        for (int k = b0; k < b1; ++k) sum += cache[k];
-        int run = sum;  // this lane's and the lanes' past it
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int o = __shfl_down_sync(ABC_FULL, run, d);
-            if (lane + d < 32) run += o;
-        }
-        if (lane == 0) s_w[t >> 5] = run;
-        __syncthreads();
-        for (int k = (t >> 5) + 1; k < CORE_WARPS; ++k) run += s_w[k];
-        run -= sum;
-        for (int k = b1 - 1; k >= b0; --k) {
-            run += cache[k];
-            if (run >= lo + k * w) {
-                atomicMax(&s_best, k);
-                break;
-            }
-        }
-        __syncthreads();
-        lo += s_best * w;
+        lo += last_reached([&](int k) { return cache[k]; }, bins, lo, w, &s_best, s_w) * w;
         hi = min(hi, lo + w - 1);
-        __syncthreads();
     }
     if (t == 0) {
         C.val[x] = lo;
@@ -309,9 +324,168 @@ __device__ __forceinline__ void core_long(const CoreArgs &C, int32_t x, int32_t 
     __syncthreads();
 }
 
+// The rows of class 0 looked at this round, up to HUGE_BATCH at a time, by the whole grid: one block would take a row of
+// 2M entries as a chain of thousands of steps, and every round waits for it (20 such rows: k_core 127 ms, so about 24). A
+// batch goes through four phases with a barrier of the grid after each but the last: entries at or above each row's
+// value; of rows that lack some, entries by value; the new values, a block a row; marks. No other row is looked at
+// before the last phase, so the values read in the first two stand still.
+struct HugeRows {
+    int64_t s[HUGE_BATCH];
+    int32_t x[HUGE_BATCH], pre[HUGE_BATCH + 1];  // (pre: chunks of the rows before it)
+};
+
+__device__ __forceinline__ void huge_load(const CoreArgs &C, HugeRows &H, const int32_t *rows, int n) {
+    __shared__ int s_w[CORE_WARPS];
+    static_assert(HUGE_BATCH == CORE_THREADS, "a thread a row");
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int nc = 0;
+    __syncthreads();
+    if (t < n) {
+        const int32_t x = __ldcg(&rows[t]);
+        const int64_t s = __ldg(&C.off[x]);
+        nc = (int)((__ldg(&C.off[x + 1]) - s + HUGE_CHUNK - 1) / HUGE_CHUNK);
+        H.s[t] = s;
+        H.x[t] = x;
+    }
+    int inc = abc::warp_incl_scan(nc);
+    if (lane == 31) s_w[w] = inc;
+    __syncthreads();
+    for (int k = 0; k < w; ++k) inc += s_w[k];
+    H.pre[t + 1] = inc;
+    if (t == 0) H.pre[0] = 0;
+    __syncthreads();
+}
+
+// fn(row of the batch, its vertex, y[], v[]) on the entries below the row's bound, four a thread at a time (y = -1: none; the
+// warp is together); before(row) says up to which id its entries can count (0: nothing is asked of it), after(row) follows each
+// chunk. Block-collective.
+template <class B, class F, class A>
+__device__ __forceinline__ void huge_walk(const CoreArgs &C, const HugeRows &H, int n, B bound_of, F fn, A after) {
+    constexpr int HILP = 4;
+    const int all = H.pre[n];
+    for (int k = blockIdx.x; k < all; k += gridDim.x) {
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (H.pre[mid] <= k) lo = mid;
+            else hi = mid - 1;
+        }
+        const int32_t x = H.x[lo], bound = bound_of(lo, x);
+        if (bound == 0) continue;
+        const int64_t f = __ldg(&C.off[x + 1]), p0 = H.s[lo] + (int64_t)(k - H.pre[lo]) * HUGE_CHUNK, p1 = min(p0 + HUGE_CHUNK, f);
+        if (__ldg(&C.adj[p0]) >= bound) continue;
+        for (int64_t p = p0; p < p1; p += CORE_THREADS * HILP) {
+            int32_t y[HILP], v[HILP];
+#pragma unroll
+            for (int q = 0; q < HILP; ++q) {
+                const int64_t e = p + q * CORE_THREADS + threadIdx.x;
+                y[q] = e < p1 ? __ldg(&C.adj[e]) : -1;
+                if (y[q] >= bound) y[q] = -1;
+            }
+#pragma unroll
+            for (int q = 0; q < HILP; ++q) v[q] = y[q] >= 0 ? ld_val(&C.val[y[q]]) : -1;
+#pragma unroll
+            for (int q = 0; q < HILP; ++q) fn(lo, x, y[q], v[q]);
+        }
+        after(lo, x);
+    }
+}
+
+// Returns false if the grid saw an error.
+__device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const int32_t *rows, int n, int32_t *cache, CoreBuf &b, int &nb,
+                                          int32_t *next, unsigned *count) {
+    __shared__ int s_best, s_w[CORE_WARPS];
+    const int t = threadIdx.x, lane = t & 31, G = gridDim.x;
+    huge_load(C, H, rows, n);
+    if (blockIdx.x == 0 && t < n) C.queued[H.x[t]] = 0;  // (nothing is lowered, and so nothing marked, before the next barrier)
+    // entries at or above the value
+    int mine = 0, e = 0;
+    huge_walk(C, H, n, [&](int, int32_t x) { return id_bound(C, x < C.nU, e = ld_val(&C.val[x])); },
+              [&](int, int32_t, int32_t, int32_t v) { mine += v >= e ? 1 : 0; },
+              [&](int r, int32_t) {
+                  mine = __reduce_add_sync(ABC_FULL, mine);
+                  if (lane == 0 && mine) atomicAdd(&C.hcnt[r], mine);
+                  mine = 0;
+              });
+    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return false;
+    // of rows that lack some: entries by value, in steps of w over [c, e)
+    auto step = [&](int c, int e) { return (e - 1 - c + CORE_CACHE) / CORE_CACHE; };
+    int c = 0, w = 1;
+    int held = -1;  // the row whose counts the block holds
+    auto write_back = [&]() {
+        if (held < 0) return;
+        __syncthreads();
+        for (int k = t; k < CORE_CACHE; k += CORE_THREADS)
+            if (cache[k]) {
+                atomicAdd(&C.hist[(int64_t)held * CORE_CACHE + k], cache[k]);
+                cache[k] = 0;
+            }
+        held = -1;
+        __syncthreads();
+    };
+    for (int k = t; k < CORE_CACHE; k += CORE_THREADS) cache[k] = 0;
+    __syncthreads();
+    huge_walk(C, H, n,
+              [&](int r, int32_t x) {
+                  e = ld_val(&C.val[x]);
+                  c = __ldcg(&C.hcnt[r]);
+                  if (c >= e) return 0;
+                  w = step(c, e);
+                  if (held != r) write_back();
+                  held = r;
+                  return id_bound(C, x < C.nU, max(c, 1));
+              },
+              [&](int, int32_t, int32_t, int32_t v) {
+                  // (most are at the top or below it all; those at the top are counted in registers)
+                  if (v >= e - 1) ++mine;
+                  else if (v >= c) atomicAdd(&cache[(v - c) / w], 1);
+              },
+              [&](int, int32_t) {
+                  mine = __reduce_add_sync(ABC_FULL, mine);
+                  if (lane == 0 && mine) atomicAdd(&cache[(e - 1 - c) / w], mine);
+                  mine = 0;
+              });
+    write_back();
+    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return false;
+    // the new values, a block a row. Where a step is several values its last one is taken, which is not too low, and the row
+    // is looked at again.
+    for (int r = blockIdx.x; r < n; r += G) {
+        const int32_t x = H.x[r];
+        e = ld_val(&C.val[x]);
+        c = __ldcg(&C.hcnt[r]);
+        int nv = -1;
+        if (c < e) {
+            w = step(c, e);
+            const int bins = (e - 1 - c) / w + 1;
+            int32_t *h = C.hist + (int64_t)r * CORE_CACHE;
+            nv = min(e - 1, c + last_reached([&](int k) { return __ldcg(&h[k]); }, bins, c, w, &s_best, s_w) * w + w - 1);
+            for (int k = t; k < bins; k += CORE_THREADS) h[k] = 0;
+            if (t < 32) core_mark(C, b, nb, t == 0 && w > 1, x, next, count);
+        }
+        __syncthreads();
+        if (t == 0) {
+            if (nv >= 0) C.val[x] = nv;
+            C.hval[r] = nv;
+            C.hcnt[r] = 0;
+        }
+        __syncthreads();
+    }
+    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return false;
+    // neighbours above a new value may have counted the old one
+    int nv = 0;
+    huge_walk(C, H, n,
+              [&](int r, int32_t x) {
+                  nv = __ldcg(&C.hval[r]);
+                  return nv < 0 ? 0 : id_bound(C, x < C.nU, nv + 1);
+              },
+              [&](int, int32_t, int32_t y, int32_t v) { core_mark(C, b, nb, v > nv, max(y, 0), next, count); }, [&](int, int32_t) {});
+    return true;
+}
+
 __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
     __shared__ CoreBuf buf[CORE_WARPS];
     __shared__ int32_t cache[CORE_CACHE];
+    __shared__ HugeRows huge;
     const int G = gridDim.x, lane = threadIdx.x & 31;
     const int64_t n = (int64_t)C.nU + C.nV;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)G * blockDim.x;
@@ -335,33 +509,39 @@ __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
     if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
     // round 0 looks at every vertex with an edge, later rounds at the lists
     for (unsigned round = 0;; ++round) {
-        const unsigned *cnt = C.count + 3 * (round % 3);
-        unsigned *ncnt = C.count + 3 * ((round + 1) % 3);
-        const int32_t *cur = C.list[round & 1];
+        const unsigned *cnt = C.count + CLASSES * (round % 3);
+        unsigned *ncnt = C.count + CLASSES * ((round + 1) % 3);
+        int32_t *cur = C.list[round & 1];
         int32_t *next = C.list[(round + 1) & 1];
-        int64_t num[3];
-        if (round == 0) {
-            num[0] = (int64_t)C.hU[0] + C.hV[0];
-            num[1] = (int64_t)(C.hU[1] - C.hU[0]) + (C.hV[1] - C.hV[0]);
-            num[2] = (int64_t)(C.zU - C.hU[1]) + (C.zV - C.hV[1]);
-        } else {
-            for (int c = 0; c < 3; ++c) num[c] = __ldcg(&cnt[c]);
-            if (num[0] + num[1] + num[2] == 0) break;
+        int64_t num[CLASSES], sum = 0;
+        for (int c = 0; c < CLASSES; ++c) {
+            num[c] = round > 0 ? (int64_t)__ldcg(&cnt[c])
+                               : (int64_t)(C.hU[c] - (c ? C.hU[c - 1] : 0)) + (C.hV[c] - (c ? C.hV[c - 1] : 0));
+            sum += num[c];
         }
+        if (sum == 0) break;
         if (t0 == 0) {  // (nothing uses this third of the counts before the round's barrier)
-            unsigned *z = C.count + 3 * ((round + 2) % 3);
-            z[0] = z[1] = z[2] = 0;
+            unsigned *z = C.count + CLASSES * ((round + 2) % 3);
+            for (int c = 0; c < CLASSES; ++c) z[c] = 0;
         }
         auto pick = [&](int c, int64_t i) -> int32_t {
             if (round > 0) return __ldcg(&cur[list_start(C, c) + i]);
-            const int32_t u0 = c == 0 ? 0 : C.hU[c - 1], u1 = c == 2 ? C.zU : C.hU[c], v0 = c == 0 ? 0 : C.hV[c - 1];
+            const int32_t u0 = c == 0 ? 0 : C.hU[c - 1], u1 = C.hU[c], v0 = c == 0 ? 0 : C.hV[c - 1];
             return i < u1 - u0 ? (int32_t)(u0 + i) : (int32_t)(C.nU + v0 + (i - (u1 - u0)));
         };
-        for (int64_t i = blockIdx.x; i < num[0]; i += G) core_long(C, pick(0, i), cache, b, nb, next, ncnt);
-        for (int64_t i = gw; i < num[1]; i += nw) core_rows<32, CORE_MID / 32>(C, pick(1, i), b, nb, next, ncnt);
-        for (int64_t i = 4 * (int64_t)gw; i < num[2]; i += 4 * (int64_t)nw) {
+        if (num[0] > 0) {
+            if (round == 0) {  // the grid's rows come from the list
+                for (int64_t i = t0; i < num[0]; i += nt) cur[i] = pick(0, i);
+                if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
+            }
+            for (int64_t i = 0; i < num[0]; i += HUGE_BATCH)
+                if (!core_huge(C, huge, cur + i, (int)min((int64_t)HUGE_BATCH, num[0] - i), cache, b, nb, next, ncnt)) return;
+        }
+        for (int64_t i = blockIdx.x; i < num[1]; i += G) core_long(C, pick(1, i), cache, b, nb, next, ncnt);
+        for (int64_t i = gw; i < num[2]; i += nw) core_rows<32, CORE_MID / 32>(C, pick(2, i), b, nb, next, ncnt);
+        for (int64_t i = 4 * (int64_t)gw; i < num[3]; i += 4 * (int64_t)nw) {
             const int64_t k = i + lane / 8;
-            core_rows<8, CORE_SMALL / 8>(C, k < num[2] ? pick(2, k) : -1, b, nb, next, ncnt);
+            core_rows<8, CORE_SMALL / 8>(C, k < num[3] ? pick(3, k) : -1, b, nb, next, ncnt);
         }
         core_flush(C, b, nb, next, ncnt);
         if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
@@ -424,7 +604,8 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
     const int64_t n = std::max<int64_t>(g.n(), 1);
     ABC_TRY(peel_finish(ctx));
     ABC_TRY(peel_prepare(ctx));  // (for the queries this is the preprocessing of)
-    int32_t *words = nullptr, *tables = nullptr;
+    constexpr size_t SMALL_WORDS = 3 * CLASSES + 1 + 64, HUGE_WORDS = (size_t)HUGE_BATCH * (2 + CORE_CACHE);
+    int32_t *words = nullptr, *tables = nullptr, *huge = nullptr;
     unsigned *small = nullptr;
     PeelCtl *ctl = nullptr;
     int rc = ABCORE_OK;
@@ -446,7 +627,8 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
     } while (0)
     STEP(ctx->alloc(&words, (size_t)(4 * n), "core values"));  // values, marks, two lists
     STEP(ctx->alloc(&tables, 2 * nt, "degree tables"));
-    STEP(ctx->alloc(&small, 9 + 1 + 64, "core counters"));     // list lengths, largest core number, barrier
+    STEP(ctx->alloc(&small, SMALL_WORDS, "core counters"));    // list lengths, largest core number, barrier
+    if (maxdeg > CORE_LONG) STEP(ctx->alloc(&huge, HUGE_WORDS, "core value counts"));
     STEP(ctx->alloc(&ctl, 1, "core control"));
     {
         CoreArgs C{};
@@ -454,13 +636,14 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
         C.adj = g.adj;
         C.nU = g.nU;
         C.nV = g.nV;
-        const int32_t cut[2] = {CORE_MID + 1, CORE_SMALL + 1};
-        for (int k = 0; k < 2; ++k) {
+        const int32_t cut[CLASSES] = {CORE_LONG + 1, CORE_MID + 1, CORE_SMALL + 1, 1};
+        for (int k = 0; k < CLASSES; ++k) {
             C.hU[k] = (int32_t)cnt_ge(g.cntU_ge, cut[k]);
             C.hV[k] = (int32_t)cnt_ge(g.cntV_ge, cut[k]);
         }
-        C.zU = (int32_t)cnt_ge(g.cntU_ge, 1);
-        C.zV = (int32_t)cnt_ge(g.cntV_ge, 1);
+        C.hcnt = huge;
+        C.hval = huge + HUGE_BATCH;
+        C.hist = huge + 2 * HUGE_BATCH;
         C.gU = tables;
         C.gV = tables + nt;
         C.maxdeg = maxdeg;
@@ -470,7 +653,7 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
         C.list[1] = words + 3 * n;
         C.count = small;
         C.ctl = ctl;
-        C.bar = small + 10;
+        C.bar = small + 3 * CLASSES + 1;
         C.timeout_ns = (unsigned long long)ctx->prm.timeout_ms * 1000000ull;
         void *args[] = {&C};
         cudaLaunchConfig_t cfg{};
@@ -485,15 +668,16 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
         const unsigned gi = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)ctx->num_sms * 8);
         int err = 0, largest = 0;
         cudaError_t e = cudaMemcpyAsync(tables, h.data(), sizeof(int32_t) * h.size(), cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(small, 0, (9 + 1 + 64) * sizeof(unsigned), ctx->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(small, 0, SMALL_WORDS * sizeof(unsigned), ctx->stream);
+        if (e == cudaSuccess && huge) e = cudaMemsetAsync(huge, 0, HUGE_WORDS * sizeof(int32_t), ctx->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(ctl, 0, sizeof(PeelCtl), ctx->stream);
         if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, (const void *)k_core, args);
         if (e == cudaSuccess) {
             ctx->stats.launches++;
-            k_core_by_caller<<<gi, 256, 0, ctx->stream>>>(C.val, g.new2old, g.nU, g.n(), core_caller, (int *)small + 9);
+            k_core_by_caller<<<gi, 256, 0, ctx->stream>>>(C.val, g.new2old, g.nU, g.n(), core_caller, (int *)small + 3 * CLASSES);
             e = cudaMemcpyAsync(&err, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&largest, small + 9, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&largest, small + 3 * CLASSES, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
         if (e != cudaSuccess) STEP(ctx->cuda_fail(e, "core decomposition"));
         if (err) STEP(ctx->fail(err, "core decomposition: device error %d", err));
@@ -504,6 +688,7 @@ done:
     ctx->release(words);
     ctx->release(tables);
     ctx->release(small);
+    ctx->release(huge);
     ctx->release(ctl);
     return rc;
 #undef STEP

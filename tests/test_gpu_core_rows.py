@@ -34,19 +34,35 @@ def _check(nU, nV, eu, ev):
     core.close()
 
 
-@pytest.mark.parametrize("per", [513, 514, 769, 4095, 4096, 4097, 20_000, 66_000])
+@pytest.mark.parametrize("per", [513, 514, 769, 4095, 4096, 4097, 20_000, 32_768, 32_769, 36_865, 66_000])
 def test_hubs_among_an_ordinary_graph(per):
     _check(*_with_hubs(7, per, 40_000, 70_000, 900_000, per))
 
 
-def test_a_row_whose_value_falls_by_thousands():
+@pytest.mark.parametrize("more", [0, 30_000])
+def test_a_row_whose_value_falls_by_thousands(more):
     # a hub whose 4,600 neighbours have 4,400 others each, all of low degree: its first value is 4,401, its core number 2
+    # (with 30,000 more of degree 1 its row is one of those the whole grid takes)
     hubs, leaves = 4600, 4400
     pool = hubs * leaves // 2
     k = np.random.default_rng(1).permutation(hubs * leaves)
     lu, lv = (k % pool).astype(np.int32), (k // leaves).astype(np.int32)  # (a leaf twice at most, at different hubs)
-    nU, nV = pool + 1, hubs
-    _check(nU, nV, np.concatenate([lu, np.full(hubs, pool, np.int32)]), np.concatenate([lv, np.arange(hubs, dtype=np.int32)]))
+    nU, nV = pool + 1, hubs + more
+    _check(nU, nV, np.concatenate([lu, np.full(nV, pool, np.int32)]), np.concatenate([lv, np.arange(nV, dtype=np.int32)]))
+
+
+@pytest.mark.parametrize("k", [255, 256, 257, 300])
+def test_more_rows_of_the_grid_than_a_batch(k):
+    # k rows of 33,000 or so in one layer, some of them neighbours of two such rows in the other
+    rng = np.random.default_rng(k)
+    nV = 34_000
+    u = np.repeat(np.arange(k, dtype=np.int32), nV)
+    v = np.tile(np.arange(nV, dtype=np.int32), k)
+    keep = rng.random(len(u)) < 0.975
+    extra = np.arange(40_000, dtype=np.int32) + k  # the upper layer's other vertices: two lower hubs reach them
+    eu = np.concatenate([u[keep], extra, extra])
+    ev = np.concatenate([v[keep], np.full(40_000, 5, np.int32), np.full(40_000, 7, np.int32)])
+    _check(k + 40_000, nV, eu, ev)
 
 
 def test_hubs_take_no_longer_than_building_the_graph_does():
