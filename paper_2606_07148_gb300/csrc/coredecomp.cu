@@ -38,6 +38,8 @@ constexpr int CORE_SMALL = 64, CORE_MID = 512, CORE_LONG = 32768;
 constexpr int CLASSES = 4;        // 0: the longest
 constexpr int CORE_CACHE = 4096;  // values of a long row a block keeps in shared memory
 constexpr int CORE_BUF = 128;     // vertices a warp collects before it adds them to a list
+constexpr int NARROW = 64;        // lists of up to this many short rows are left to one block (core_narrow), which
+constexpr int NARROW_MAX = 256;   // goes on with what those mark while it is not more than this
 constexpr int HUGE_BATCH = 256;   // rows of class 0 the grid takes together
 constexpr int HUGE_CHUNK = 4096;  // entries of one a block takes at a time
 
@@ -482,6 +484,108 @@ __device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const 
     return true;
 }
 
+// Rounds of few short rows, by one block while the grid waits once: a round of the grid takes about 20 us, mostly
+// its barrier and the lists, whatever it has to look at, and a change moves on by one neighbour a round, so a path of n
+// vertices needs about n / 2 rounds. Here the lists stay in shared memory, with the rows' places (read while the
+// mark is made), and a round is three trips to L2 and two block barriers. Rounds end when nothing is left, when a
+// longer row is marked or the list is full, or after `rounds`; what is left goes to the grid's list.
+struct NarrowList {
+    int64_t s[NARROW_MAX];
+    int32_t x[NARROW_MAX], len[NARROW_MAX];
+};
+static_assert(2 * sizeof(NarrowList) <= CORE_CACHE * sizeof(int32_t), "the lists lie in the cache");
+
+__device__ __forceinline__ void core_narrow(const CoreArgs &C, const int32_t *rows, int n, int32_t *cache, int32_t *next, unsigned *count, int rounds) {
+    __shared__ int s_cnt[2], s_spilt;
+    NarrowList *const L = reinterpret_cast<NarrowList *>(cache);
+    constexpr int W = 8, R = CORE_SMALL / W;
+    const int t = threadIdx.x, lane = t & 31, gl = lane % W;
+    const unsigned group = ((1u << W) - 1u) << (lane - gl);
+    if (t < n) {
+        const int32_t x = __ldcg(&rows[t]);
+        const int64_t s = __ldg(&C.off[x]);
+        L[0].x[t] = x;
+        L[0].s[t] = s;
+        L[0].len[t] = (int32_t)(__ldg(&C.off[x + 1]) - s);
+    }
+    if (t == 0) {
+        s_cnt[1] = 0;
+        s_spilt = 0;
+    }
+    __syncthreads();
+    int a = 0;
+    for (int round = 0; n > 0; ++round) {
+        NarrowList &cur = L[a], &nxt = L[a ^ 1];
+        for (int i0 = 0; i0 < n; i0 += CORE_THREADS / W) {
+            const int i = i0 + t / W;
+            const int32_t x = i < n ? cur.x[i] : -1;
+            const int64_t s = i < n ? cur.s[i] : 0;
+            const int len = i < n ? cur.len[i] : 0;
+            const int e = x >= 0 ? ld_val(&C.val[x]) : 0;
+            int most = len;
+#pragma unroll
+            for (int d = 16; d >= W; d >>= 1) most = max(most, __shfl_xor_sync(ABC_FULL, most, d));
+            const int nr = (most + W - 1) / W;  // the same for the warp
+            int32_t y[R], v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                y[r] = -1;
+                if (r < nr && r * W + gl < len) y[r] = __ldg(&C.adj[s + r * W + gl]);
+            }
+            if (x >= 0 && gl == 0) C.queued[x] = 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = y[r] >= 0 ? ld_val(&C.val[y[r]]) : -1;
+            auto at_least = [&](int k) {
+                int c = 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (r < nr) c += __popc(__ballot_sync(ABC_FULL, v[r] >= k) & group);
+                return c;
+            };
+            const int c = at_least(e);
+            const bool drops = x >= 0 && c < e;
+            int lo = drops ? c : 0, hi = drops ? e - 1 : 0;
+            while (__ballot_sync(ABC_FULL, lo < hi)) {
+                const int mid = lo + ((hi - lo + 1) >> 1);
+                const int k = at_least(mid);
+                if (lo < hi) {
+                    if (k >= mid) lo = mid;
+                    else hi = mid - 1;
+                }
+            }
+            // (all of them have read and cleared their marks: what is lowered and marked from here on is seen by whoever is next)
+            __syncthreads();
+            if (drops && gl == 0) C.val[x] = lo;
+            if (drops) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (v[r] <= lo) continue;
+                    const int64_t f = __ldg(&C.off[y[r]]), g = __ldg(&C.off[y[r] + 1]);
+                    if (atomicExch(&C.queued[y[r]], 1) != 0) continue;
+                    const int at = g - f <= CORE_SMALL ? atomicAdd(&s_cnt[a ^ 1], 1) : NARROW_MAX;
+                    if (at < NARROW_MAX) {
+                        nxt.x[at] = y[r];
+                        nxt.s[at] = f;
+                        nxt.len[at] = (int32_t)(g - f);
+                    } else {
+                        const int k = row_class(C, y[r]);
+                        next[list_start(C, k) + atomicAdd(&count[k], 1u)] = y[r];
+                        s_spilt = 1;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        a ^= 1;
+        n = min(s_cnt[a], NARROW_MAX);
+        const bool leave = s_spilt != 0 || round + 1 >= rounds;
+        if (t == 0) s_cnt[a ^ 1] = 0;  // (added to after the next barrier only)
+        if (leave) break;
+    }
+    if (t < n) next[list_start(C, CLASSES - 1) + atomicAdd(&count[CLASSES - 1], 1u)] = L[a].x[t];
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
     __shared__ CoreBuf buf[CORE_WARPS];
     __shared__ int32_t cache[CORE_CACHE];
@@ -529,6 +633,13 @@ __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
             const int32_t u0 = c == 0 ? 0 : C.hU[c - 1], u1 = C.hU[c], v0 = c == 0 ? 0 : C.hV[c - 1];
             return i < u1 - u0 ? (int32_t)(u0 + i) : (int32_t)(C.nU + v0 + (i - (u1 - u0)));
         };
+        if (round > 0 && sum == num[CLASSES - 1] && sum <= NARROW) {
+            // (a round of it takes up to 10 us; the other blocks' wait has its limit)
+            if (blockIdx.x == 0)
+                core_narrow(C, cur + list_start(C, CLASSES - 1), (int)sum, cache, next, ncnt, (int)max(16ull, min(4096ull, C.timeout_ns / 20000ull)));
+            if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
+            continue;
+        }
         if (num[0] > 0) {
             if (round == 0) {  // the grid's rows come from the list
                 for (int64_t i = t0; i < num[0]; i += nt) cur[i] = pick(0, i);
