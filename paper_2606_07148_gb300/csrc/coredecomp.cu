@@ -9,8 +9,12 @@
 // Seshadhri and Pinar, "Local algorithms for hierarchical dense subgraph discovery", 2018). A peel
 // goes through every k and every cascade level inside it, one after the other: on a 20M-edge power-law graph
 // 1,322 levels of a few vertices each, 15.9 ms of latency. The h-index rounds need up to 60 there and the
-// work of about eight passes over the edges, most of it in the first, wide rounds: 3.1 ms, bound by
-// the latency of the later rounds' long rows and barriers.
+// work of about eight passes over the edges, most of it in the first, wide rounds: 3.1 ms. How many rounds there are
+// depends on how deep the graph is, since a change moves on by one neighbour a round: a path of n vertices
+// has about n / 2. A grid round takes about 10 us whatever its lists hold (barrier, lists, one row's trips to L2), so
+// rounds of a few short rows are left to one block (core_narrow), and rows that would hold up a round to
+// the whole grid (core_huge). Whole calls, peel of every k / rounds: path of 200,000 vertices 281 / 165 ms, 1,000 x 1,000 grid
+// 9.3 / 10.0, 300 x 300 2.96 / 3.06, 20 rows of 2M entries 98 / 60, 300M edges 176 / 60.
 //
 // Rows ascend in degree order, which bounds what is read: a vertex's first value is the h-index of its
 // neighbours' degrees, a binary search in its row; and a neighbour can count for t only if its degree is
@@ -40,6 +44,7 @@ constexpr int CORE_CACHE = 4096;  // values of a long row a block keeps in share
 constexpr int CORE_BUF = 128;     // vertices a warp collects before it adds them to a list
 constexpr int NARROW = 64;        // lists of up to this many short rows are left to one block (core_narrow), which
 constexpr int NARROW_MAX = 256;   // goes on with what those mark while it is not more than this
+constexpr int EAGER = 1 << 16;    // see core_mark
 constexpr int HUGE_BATCH = 256;   // rows of class 0 the grid takes together
 constexpr int HUGE_CHUNK = 4096;  // entries of one a block takes at a time
 
@@ -57,9 +62,41 @@ struct CoreArgs {
     int32_t *hcnt, *hval, *hist;    // [HUGE_BATCH] of a batch of class 0: entries at or above the value, the new value or -1;
                                     // [HUGE_BATCH][CORE_CACHE] entries by value
     PeelCtl *ctl;
-    unsigned *bar;
+    unsigned long long *bar;        // blocks arrived at the grid's barriers so far
     unsigned long long timeout_ns;
 };
+
+// Barrier of the grid, the `passed`-th (counted here): one count that only grows, looked at without reading the clock at
+// first. A deep graph goes through hundreds of rounds with little to do between them (a grid of 1,000 x 1,000: 500), and
+// the general group barrier, with its two words, its fixup and a clock reading per look, was half of each. Returns
+// false if the session saw an error, in which case every block leaves. Block-collective.
+__device__ __forceinline__ bool core_barrier(const CoreArgs &C, unsigned long long &passed) {
+    __shared__ int s_ok;
+    __syncthreads();
+    const unsigned long long all = ++passed * gridDim.x;
+    if (threadIdx.x == 0) {
+        s_ok = 1;
+        __threadfence();
+        if (atomicAdd(C.bar, 1ull) + 1 < all) {
+            int looks = 0;
+            unsigned long long t0 = 0;
+            while (abc::ld_acquire(C.bar) < all) {
+                if (++looks < 64) continue;
+                const unsigned long long now = abc::now_ns();
+                if (t0 == 0) t0 = now;
+                if (now - t0 > C.timeout_ns) abc::set_error(&C.ctl->err, ABCORE_ETIMEDOUT);
+                if (abc::ld_relaxed_i32(&C.ctl->err) != 0) {
+                    s_ok = 0;
+                    break;
+                }
+                __nanosleep(256);
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
 
 __device__ __forceinline__ int32_t ld_val(const int32_t *p) {
     int32_t v;
@@ -110,10 +147,12 @@ __device__ __forceinline__ void core_flush(const CoreArgs &C, CoreBuf &b, int &n
     nb = 0;
 }
 
-// Warp-collective: lanes with `want` have neighbour y to look at again.
-__device__ __forceinline__ void core_mark(const CoreArgs &C, CoreBuf &b, int &nb, bool want, int32_t y, int32_t *next, unsigned *count) {
+// Warp-collective: lanes with `want` have neighbour y to look at again. `eager`: the word is not read before it is
+// exchanged, a trip to L2 less in rounds of few rows (many rows marking the same vertices would all write it).
+__device__ __forceinline__ void core_mark(const CoreArgs &C, CoreBuf &b, int &nb, bool want, int32_t y, int32_t *next, unsigned *count,
+                                          bool eager = false) {
     // (a vertex still waiting to be looked at will see the new value: the word is cleared before the values are read)
-    const bool add = want && ld_val(&C.queued[y]) == 0 && atomicExch(&C.queued[y], 1) == 0;
+    const bool add = want && (eager || ld_val(&C.queued[y]) == 0) && atomicExch(&C.queued[y], 1) == 0;
     const unsigned m = __ballot_sync(ABC_FULL, add);
     if (m == 0) return;
     if (add) b.x[nb + __popc(m & abc::lanemask_lt())] = y;
@@ -124,7 +163,7 @@ __device__ __forceinline__ void core_mark(const CoreArgs &C, CoreBuf &b, int &nb
 // Rows of up to W * R entries, W lanes each, all values in registers: every group of W lanes lowers its vertex x
 // (x < 0: none) to the h-index of its neighbours' values. Warp-collective.
 template <int W, int R>
-__device__ __forceinline__ void core_rows(const CoreArgs &C, int32_t x, CoreBuf &b, int &nb, int32_t *next, unsigned *count) {
+__device__ __forceinline__ void core_rows(const CoreArgs &C, int32_t x, CoreBuf &b, int &nb, int32_t *next, unsigned *count, bool eager) {
     const int lane = threadIdx.x & 31, gl = lane % W;
     const unsigned group = W == 32 ? ABC_FULL : ((1u << (W & 31)) - 1u) << (lane / W * W);
     int64_t s = 0;
@@ -177,7 +216,7 @@ __device__ __forceinline__ void core_rows(const CoreArgs &C, int32_t x, CoreBuf 
     // neighbours above the new value may have counted this one (v was read before: it can only be too high)
 #pragma unroll
     for (int r = 0; r < R; ++r)
-        if (r < nr) core_mark(C, b, nb, drops && v[r] > lo, y[r], next, count);
+        if (r < nr) core_mark(C, b, nb, drops && v[r] > lo, y[r], next, count, eager);
 }
 
 // How many of the ascending entries adj[s, f) are below `bound`: every thread probes a place, which cuts the row in 257.
@@ -395,7 +434,7 @@ __device__ __forceinline__ void huge_walk(const CoreArgs &C, const HugeRows &H, 
 
 // Returns false if the grid saw an error.
 __device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const int32_t *rows, int n, int32_t *cache, CoreBuf &b, int &nb,
-                                          int32_t *next, unsigned *count) {
+                                          int32_t *next, unsigned *count, unsigned long long &passed) {
     __shared__ int s_best, s_w[CORE_WARPS];
     const int t = threadIdx.x, lane = t & 31, G = gridDim.x;
     huge_load(C, H, rows, n);
@@ -409,7 +448,7 @@ __device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const 
                   if (lane == 0 && mine) atomicAdd(&C.hcnt[r], mine);
                   mine = 0;
               });
-    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return false;
+    if (!core_barrier(C, passed)) return false;
     // of rows that lack some: entries by value, in steps of w over [c, e)
     auto step = [&](int c, int e) { return (e - 1 - c + CORE_CACHE) / CORE_CACHE; };
     int c = 0, w = 1;
@@ -448,7 +487,7 @@ __device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const 
                   mine = 0;
               });
     write_back();
-    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return false;
+    if (!core_barrier(C, passed)) return false;
     // the new values, a block a row. Where a step is several values its last one is taken, which is not too low, and the row
     // is looked at again.
     for (int r = blockIdx.x; r < n; r += G) {
@@ -472,7 +511,7 @@ __device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const 
         }
         __syncthreads();
     }
-    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return false;
+    if (!core_barrier(C, passed)) return false;
     // neighbours above a new value may have counted the old one
     int nv = 0;
     huge_walk(C, H, n,
@@ -484,8 +523,8 @@ __device__ __forceinline__ bool core_huge(const CoreArgs &C, HugeRows &H, const 
     return true;
 }
 
-// Rounds of few short rows, by one block while the grid waits once: a round of the grid takes about 20 us, mostly
-// its barrier and the lists, whatever it has to look at, and a change moves on by one neighbour a round, so a path of n
+// Rounds of few short rows, by one block while the grid waits once: a round of the grid takes about 10 us (20
+// when this was made), mostly its barrier and the lists, whatever it has to look at, and a change moves on by one neighbour a round, so a path of n
 // vertices needs about n / 2 rounds. Here the lists stay in shared memory, with the rows' places (read while the
 // mark is made), and a round is three trips to L2 and two block barriers. Rounds end when nothing is left, when a
 // longer row is marked or the list is full, or after `rounds`; what is left goes to the grid's list.
@@ -596,6 +635,7 @@ __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
     const int gw = (int)(t0 >> 5), nw = (int)(nt >> 5);
     CoreBuf &b = buf[threadIdx.x >> 5];
     int nb = 0;
+    unsigned long long passed = 0;
 
     // first values: the largest h whose h-th entry has at least h edges
     for (int64_t x = t0; x < n; x += nt) {
@@ -610,13 +650,16 @@ __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
         C.val[x] = lo;
         C.queued[x] = 1;
     }
-    if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
+    if (!core_barrier(C, passed)) return;
     // round 0 looks at every vertex with an edge, later rounds at the lists
     for (unsigned round = 0;; ++round) {
         const unsigned *cnt = C.count + CLASSES * (round % 3);
         unsigned *ncnt = C.count + CLASSES * ((round + 1) % 3);
         int32_t *cur = C.list[round & 1];
         int32_t *next = C.list[(round + 1) & 1];
+        // a first short row per eight lanes, read along with the counts that say whether there is one
+        const int64_t at0 = 4 * (int64_t)gw + lane / 8, short0 = list_start(C, CLASSES - 1), shorts = (int64_t)C.hU[CLASSES - 1] + C.hV[CLASSES - 1] - short0;
+        const int32_t first = round > 0 && at0 < shorts ? __ldcg(&cur[short0 + at0]) : -1;
         int64_t num[CLASSES], sum = 0;
         for (int c = 0; c < CLASSES; ++c) {
             num[c] = round > 0 ? (int64_t)__ldcg(&cnt[c])
@@ -637,25 +680,25 @@ __global__ void __launch_bounds__(CORE_THREADS, 4) k_core(CoreArgs C) {
             // (a round of it takes up to 10 us; the other blocks' wait has its limit)
             if (blockIdx.x == 0)
                 core_narrow(C, cur + list_start(C, CLASSES - 1), (int)sum, cache, next, ncnt, (int)max(16ull, min(4096ull, C.timeout_ns / 20000ull)));
-            if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
+            if (!core_barrier(C, passed)) return;
             continue;
         }
         if (num[0] > 0) {
             if (round == 0) {  // the grid's rows come from the list
                 for (int64_t i = t0; i < num[0]; i += nt) cur[i] = pick(0, i);
-                if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
+                if (!core_barrier(C, passed)) return;
             }
             for (int64_t i = 0; i < num[0]; i += HUGE_BATCH)
-                if (!core_huge(C, huge, cur + i, (int)min((int64_t)HUGE_BATCH, num[0] - i), cache, b, nb, next, ncnt)) return;
+                if (!core_huge(C, huge, cur + i, (int)min((int64_t)HUGE_BATCH, num[0] - i), cache, b, nb, next, ncnt, passed)) return;
         }
         for (int64_t i = blockIdx.x; i < num[1]; i += G) core_long(C, pick(1, i), cache, b, nb, next, ncnt);
-        for (int64_t i = gw; i < num[2]; i += nw) core_rows<32, CORE_MID / 32>(C, pick(2, i), b, nb, next, ncnt);
+        for (int64_t i = gw; i < num[2]; i += nw) core_rows<32, CORE_MID / 32>(C, pick(2, i), b, nb, next, ncnt, sum <= EAGER);
         for (int64_t i = 4 * (int64_t)gw; i < num[3]; i += 4 * (int64_t)nw) {
             const int64_t k = i + lane / 8;
-            core_rows<8, CORE_SMALL / 8>(C, k < num[3] ? pick(3, k) : -1, b, nb, next, ncnt);
+            core_rows<8, CORE_SMALL / 8>(C, k >= num[3] ? -1 : round > 0 && k == at0 ? first : pick(3, k), b, nb, next, ncnt, sum <= EAGER);
         }
         core_flush(C, b, nb, next, ncnt);
-        if (!abc::group_barrier(C.bar, G, C.ctl, false, C.timeout_ns)) return;
+        if (!core_barrier(C, passed)) return;
     }
 }
 
@@ -715,7 +758,7 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
     const int64_t n = std::max<int64_t>(g.n(), 1);
     ABC_TRY(peel_finish(ctx));
     ABC_TRY(peel_prepare(ctx));  // (for the queries this is the preprocessing of)
-    constexpr size_t SMALL_WORDS = 3 * CLASSES + 1 + 64, HUGE_WORDS = (size_t)HUGE_BATCH * (2 + CORE_CACHE);
+    constexpr size_t BAR_WORD = (3 * CLASSES + 1 + 31) / 32 * 32, SMALL_WORDS = BAR_WORD + 2, HUGE_WORDS = (size_t)HUGE_BATCH * (2 + CORE_CACHE);
     int32_t *words = nullptr, *tables = nullptr, *huge = nullptr;
     unsigned *small = nullptr;
     PeelCtl *ctl = nullptr;
@@ -764,7 +807,7 @@ static int core_decompose(abcore_ctx *ctx, int32_t *core_caller, int32_t *maxcor
         C.list[1] = words + 3 * n;
         C.count = small;
         C.ctl = ctl;
-        C.bar = small + 3 * CLASSES + 1;
+        C.bar = reinterpret_cast<unsigned long long *>(small + BAR_WORD);
         C.timeout_ns = (unsigned long long)ctx->prm.timeout_ms * 1000000ull;
         void *args[] = {&C};
         cudaLaunchConfig_t cfg{};
