@@ -329,12 +329,12 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *                       batch: 2 selects the batch kernel compiled for two blocks an SM).
  *   "chunk"* [1024]     adjacency entries per work item (32..2^20).
  *   "grab_div"* [0]     queue items per grab = backlog / grab_div, 1..32 (0: half the resident warps, or
- *                       all of them after a long first round or with one large bound).
+ *                       all of them after a walked first round or with few rows in it).
  *   "batch_entries"* [1024] entries a warp walks per batch (128..2^24; the rest is re-queued).
  *   "batch_entries_small"* [512] the limit when a warp's grab leaves the queue nearly empty (0 off).
  *   "local_rounds" [256] batches a warp may chain on its own pushes (0..4096).
  *   "flush_steps"* [-1] steps a buffered push may wait before its warp flushes (1..2^20); -1: by query
- *                       (16, for single peels of large bounds 1).
+ *                       (16, for single peels of large bounds and long rows 1).
  * Batch:
  *   "batch_wave"* [-1]  chains per wave (0..32; 0: all at once); -1: 4, 8 or 16 by the graph's size, and
  *                       read as that number.

@@ -136,12 +136,12 @@ struct Params {
     int chunk = 1024;
     int batch_entries = 1024;  // see PeelArgs (1024 kept a 94k-candidate, 18-level cascade 4.5x
                                // faster than 4096; the autotuner may raise it)
-    int flush_steps = -1;      // -1: by the query's bounds in a single peel (peel_compute), else 16
+    int flush_steps = -1;      // -1: by the query in a single peel (peel_compute), else 16
     int packed_counts = 1;     // batch chains keep 16-bit counts when every degree fits
     int round0 = -1;           // single peel: walk the initial candidate violators' rows with
                                // no-return atomics when a layer counts by search (k_round0), instead
                                // of queueing them; -1: where that saves enough
-                               // (first_round_entries)
+                               // (first_round)
     int round0_variant = -1;   // k_round0's compiled (entries per lane per step, blocks per SM) pair;
                                // -1: 4 or 5 by the length of the walk where round0
                                // is -1 too, else 0. 0 (8, any), 1 (4, 8), 2 (16, 4), 3 (8, 8); 4: rows four at a time;
@@ -152,7 +152,7 @@ struct Params {
     int pdl = 1;               // single peel: launch the kernels after the count init as
                                // programmatic dependents of the one before (each waits for its
                                // predecessor on the device; the launch latency overlaps its tail)
-    int grab_div = 0;          // 0 = automatic (see peel_compute)
+    int grab_div = 0;          // 0 = automatic (see ALL_WARPS_ROWS, peel.cu)
     int local_rounds = 256;    // single peel: see PeelArgs::local_rounds
     int batch_entries_small = 512; // single peel: see PeelArgs::batch_entries_small (0: off)
     int threads = 256;

@@ -48,23 +48,34 @@ constexpr int64_t SMALL_QUERY_VERTICES = 1 << 14, SMALL_QUERY_ENTRIES = 1 << 19;
 // 16 entries at once: 127 us in one block, 60 in the general peel.)
 constexpr double SMALL_QUERY_ROWS = 8192;
 
-// First rounds of at least this many entries walk the initial violators' rows without returns (unless "round0" is set)
-constexpr double ROUND0_MIN_ENTRIES = 2e6;
-// ... and no bound is above this: a walked row is shorter than its bound, and eight lanes take a long one as a chain of
-// steps while few rows are there to share. Queued / walked: 80M edges, (300,10) 411 / 462 us, (10,300) 331 / 389,
-// (112,386) 310 / 420, (500,500) 177 / 351; 300M edges, (250,30) 594 / 521, (200,200) 414 / 379, (112,386) 387 / 435.
-constexpr int ROUND0_MAX_BOUND = 256;
-// Queries whose bounds sum to more hand every push over at once and queue their first round, unless "flush_steps" and
-// "round0" are set: few vertices fall and each opens a long row. Pushes waiting one step (queued) / 16 steps (walked):
-// 80M edges, (112,386) 224 / 420 us, (250,250) 299 / 498, (500,500) 162 / 351, but (180,180) 225 / 251, (128,30) 318 /
-// 275, (20,160) 279 / 251; 300M edges, (500,500) 469 / 654, (112,386) 384 / 435, but (200,200) 428 / 379, (250,30) 639 / 521.
-constexpr int WIDE_BOUND = 128;  // see where the grab is chosen
-constexpr int64_t LONG_BOUNDS = 400;
-// ... and of at least this many with the hub table, unless the form is set: its start and its write-back are paid once,
+// What the first round is expected to be (first_round) picks how a query with both layers counted by search is peeled,
+// unless "round0", "flush_steps" and "grab_div" are set. All lines lie where a sweep of 31 pairs of bounds, (1,3) to (1000,1000), over
+// graphs of 3M, 10M, 30M, 80M and 300M edges crosses over (4,864 warps; every form of every query measured): the form picked
+// is 3 % behind the best one in the mean (rules by the bounds alone: 11 %).
+//
+// The initial violators' rows are walked without returns, or queued: the walk saves about 4.4 us a million entries and costs
+// two launches and, as a row is a chain of steps for the warp that walks it, 0.4 us an entry of the largest bound past
+// 60. Queued / walked: 80M edges, (64,64) 229 / 199 us, (100,20) 309 / 272, (160,20) 323 / 314, (20,160) 241 / 252, (300,10)
+// 362 / 429; 300M, (300,10) 1004 / 829, (200,200) 423 / 367, (500,500) 438 / 527.
+constexpr double WALK_MIN_ENTRIES = 1.4e6, WALK_ENTRIES_PER_BOUND = 0.09e6;
+constexpr int WALK_FREE_BOUND = 60;
+// Walks of at least this many take the hub table, unless the form is set: its start and its write-back are paid once,
 // and the longer the walk, the more decrements it absorbs. Whole queries, rows alone against the table: 22M entries
 // (300M edges, (30,100)) 360 / 406 us, 25M ((64,64)) 362 / 366, 46M (600M edges, (40,40), (64,64), (128,128)) 735 / 762,
 // 594 / 577, 564 / 569; 112M (1.5B edges, (64,64)) 1228 / 1143.
 constexpr double ROUND0_HUB_ENTRIES = 8e7;
+// A warp's grab is its share of what is queued, over half the warps, or over all of them after a walk (little is queued,
+// and deep) or where there are few rows and not the shortest, which half the warps would take two at a time. Half / all: 30M edges, (40,600) 597 / 216 us,
+// (401,401) 123 / 95, (180,180) 186 / 183, (300,10) 209 / 226; 10M, (100,20) 161 / 106; 80M, (10,300) 318 / 332, (20,20)
+// 261 / 283, (500,500) 144 / 150. (With an eighth of the warps the first ones took all of a short queue: 5M edges, (20,20) /
+// (40,40) 152 / 218 us, with half 71 / 81.)
+constexpr double ALL_WARPS_ENTRIES = 720, ALL_WARPS_ROWS = 32;  // (a warp)
+constexpr double SHORT_ROW = 5;
+// Pushes wait 16 steps, or, in queued rounds, one where few vertices fall and each opens a long row. 16 steps / one: 80M
+// edges, (112,386) 281 / 219 us, (500,500) 168 / 144, (40,600) 305 / 266, but (128,30) 284 / 317; 30M, (200,200) 321 / 231, (250,30)
+// 176 / 211.
+constexpr int64_t HASTY_BOUNDS = 200, HASTY_BOUNDS_ANY = 400;
+constexpr double HASTY_ROW = 23;
 constexpr int SWIZZLE_MAX_PCT = 30;  // counts are spread when candidates are less than this share of the vertices
 
 constexpr int INIT_THREADS = 256;
@@ -689,21 +700,29 @@ int pick_mode(const abcore_ctx *ctx, int32_t alpha, int32_t beta, int32_t pU, in
     return best;
 }
 
-// Row entries the first round is expected to walk when both layers count by search: a candidate of degree d has about
-// d f live candidate neighbours, f being the share of its layer's entries below the other layer's boundary, so
+// The first round as it is expected when both layers count by search, rows and their entries: a candidate of degree d has
+// about d f live candidate neighbours, f being the share of its layer's entries below the other layer's boundary, so
 // the initial violators are the candidates of degree below threshold / f.
-static double first_round_entries(const Graph &g, int32_t alpha, int32_t beta) {
+struct FirstRound {
+    double rows = 0, entries = 0;
+};
+static FirstRound first_round(const Graph &g, int32_t alpha, int32_t beta) {
     const double m = (double)std::max<int64_t>(g.m, 1);
-    auto layer = [&](int32_t thr, const std::vector<int64_t> &edges, double f) {
-        if (thr <= 0 || f <= 0.0) return 0.0;
-        const double top = std::min((double)INT32_MAX, std::ceil((double)thr / f));
-        return f * (double)(cnt_ge(edges, thr) - cnt_ge(edges, (int32_t)top));
+    FirstRound r;
+    auto layer = [&](int32_t thr, const std::vector<int64_t> &cnt, const std::vector<int64_t> &edges, double f) {
+        if (thr <= 0 || f <= 0.0) return;
+        const int32_t top = (int32_t)std::min((double)INT32_MAX, std::ceil((double)thr / f));
+        r.rows += (double)(cnt_ge(cnt, thr) - cnt_ge(cnt, top));
+        r.entries += f * (double)(cnt_ge(edges, thr) - cnt_ge(edges, top));
     };
     const double eU = (double)cnt_ge(g.edgesU_ge, alpha), eV = (double)cnt_ge(g.edgesV_ge, beta);
-    return layer(alpha, g.edgesU_ge, eV / m) + layer(beta, g.edgesV_ge, eU / m);
+    layer(alpha, g.cntU_ge, g.edgesU_ge, eV / m);
+    layer(beta, g.cntV_ge, g.edgesV_ge, eU / m);
+    return r;
 }
 
-// Rows that round is expected to have: candidates whose expected count, to the nearest whole number, misses the bound.
+// Rows the first round is expected to have where few would be surprising: candidates whose expected count, to the nearest whole
+// number, misses the bound.
 double first_round_rows(const Graph &g, int32_t alpha, int32_t beta) {
     const double m = (double)std::max<int64_t>(g.m, 1);
     auto layer = [&](int32_t thr, const std::vector<int64_t> &cnt, double f) {
@@ -823,8 +842,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     a.thrV = beta;
     a.chunk = std::max(ctx->prm.chunk, 32);
     a.batch_entries = ctx->prm.batch_entries;
-    const bool long_bounds = (int64_t)alpha + beta > LONG_BOUNDS;
-    a.flush_steps = ctx->prm.flush_steps >= 0 ? ctx->prm.flush_steps : long_bounds ? 1 : FLUSH_STEPS;
+    const FirstRound fr = first_round(ctx->g, alpha, beta);
     a.local_rounds = ctx->prm.local_rounds;
     a.batch_entries_small = ctx->prm.batch_entries_small;
     a.phases = ctx->prm.log_level >= 2 ? 1 : 0;
@@ -836,12 +854,11 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     const int blocks = cascade_grid(ctx);
     a.searchU = mode & 1;
     a.searchV = (mode >> 1) & 1;
-    // The initial violators' rows: walked first without returns, or queued. The walk and its scan cost two launches; no
-    // crossing is looked for in it, which runs half again as fast.
     int round0 = ctx->prm.round0, round0_variant = ctx->prm.round0_variant;
     if (round0 < 0) {
-        round0 = !pruned && mode == 3 && !long_bounds && std::max(alpha, beta) <= ROUND0_MAX_BOUND && first_round_entries(g, alpha, beta) >= ROUND0_MIN_ENTRIES ? 1 : 0;
-        if (round0_variant < 0) round0_variant = first_round_entries(g, alpha, beta) >= ROUND0_HUB_ENTRIES ? 5 : 4;
+        const double least = WALK_MIN_ENTRIES + WALK_ENTRIES_PER_BOUND * std::max(0, std::max(alpha, beta) - WALK_FREE_BOUND);
+        round0 = !pruned && mode == 3 && fr.entries >= least ? 1 : 0;
+        if (round0_variant < 0) round0_variant = fr.entries >= ROUND0_HUB_ENTRIES ? 5 : 4;
     }
     if (round0 && (a.searchU || a.searchV) && w.l0_cap < Pu) {
         ctx->release(w.l0);
@@ -855,15 +872,12 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
         }
     }
     a.round0 = (round0 && (a.searchU || a.searchV)) ? 1 : 0;
-    // A warp's grab: its share of what is queued. With an eighth of the warps as the divisor the first warps took all of a
-    // queue of 20,000 items, 31 each, and the tickets they held beyond it drew most later items to them
-    // too (5M edges, (20,20) / (40,40): 152 / 218 us, with half the warps 71 / 81); after a long first round
-    // what is queued is little and deep, and all warps share it.
-    // So do they with one large bound: its few rows are long (half / all warps: 10M edges, (10,300) 453 / 143 us, (300,10)
-    // 167 / 129, (180,180) 407 / 354; 80M edges, (10,300) 332 / 352, (300,10) 417 / 419, (180,180) 249 / 251).
+    const int64_t bounds = (int64_t)alpha + beta;
+    const bool hasty = !a.round0 && (bounds > HASTY_BOUNDS_ANY || (bounds > HASTY_BOUNDS && fr.entries > HASTY_ROW * fr.rows));
+    a.flush_steps = ctx->prm.flush_steps >= 0 ? ctx->prm.flush_steps : hasty ? 1 : FLUSH_STEPS;
     const int warps = blocks * (256 / 32);
-    const bool wide = !long_bounds && std::max(alpha, beta) > WIDE_BOUND;
-    a.grab_div = ctx->prm.grab_div > 0 ? ctx->prm.grab_div : std::max(1, a.round0 || wide ? warps : warps / 2);
+    const bool few = fr.rows < ALL_WARPS_ROWS * warps && fr.entries < ALL_WARPS_ENTRIES * warps && fr.entries > SHORT_ROW * fr.rows;
+    a.grab_div = ctx->prm.grab_div > 0 ? ctx->prm.grab_div : std::max(1, a.round0 || few ? warps : warps / 2);
     const bool hubs = ctx->prm.hub_degree > 0 && !pruned;
     a.hubcutU = hubs ? (int32_t)std::min<int64_t>(cnt_ge(g.cntU_ge, ctx->prm.hub_degree), pU) : 0;
     a.hubcutV = hubs ? (int32_t)std::min<int64_t>(cnt_ge(g.cntV_ge, ctx->prm.hub_degree), pV) : 0;
@@ -1048,7 +1062,7 @@ int peel_compute(abcore_ctx *ctx, int32_t alpha, int32_t beta, uint8_t *d_mask_u
     ctx->stats.mode = mode;
     ctx->stats.grid_blocks = blocks;
     ctx->log(1, "peel (%d,%d): %lld candidates, counting mode %d, first round about %.0f entries%s", alpha, beta, (long long)P, mode,
-             first_round_entries(g, alpha, beta), a.round0 ? ", walked first" : "");
+             fr.entries, a.round0 ? ", walked first" : "");
     ctx->pending_async = true;
     if (sync_and_check) return peel_finish(ctx);
     return ABCORE_OK;
