@@ -312,7 +312,9 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *   "hub_degree"* [256] rows of at least this degree always count by search (0: none).
  *   "probe_bytes"* [32] the cost model's price of a search probe (steers search vs stream).
  *   "round0"* [-1]      1: walk the initial violators' rows with no-return decrements first; 0: queue
- *                       them; -1: by query (long first rounds of short rows are walked).
+ *                       them; -1: by query (long first rounds of short rows are walked). A walk keeps a
+ *                       list of 16 bytes a candidate, made by the first query that needs it (ASYNC ones
+ *                       too); without room for it the round is queued, with 1 the query fails (ENOMEM).
  *   "round0_variant"* [-1] that walk's form: 0..3 lane-per-entry (entries in flight / blocks an SM:
  *                       8/any, 4/8, 16/4, 8/8), 4 four rows per warp, 5 the same in one 1024-thread
  *                       block per SM summing hub decrements in shared memory; -1: by query (4, for the
@@ -324,7 +326,7 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *                       percentage of the vertices, else gather over caller ids.
  *   "emit_bitmap_min_pct"* [0] the gather tests removal in a bitmap when the candidates are at
  *                       least this percentage of the vertices (101: never; by count instead).
- * Cascade (single peel; chunk, grab_div, batch_entries and flush_steps also in batch chains):
+ * Cascade (single peel; chunk, batch_entries and flush_steps also in batch chains):
  *   "blocks_per_sm"* [0] resident blocks an SM for the cascade and the batch (0: as many as fit;
  *                       batch: 2 selects the batch kernel compiled for two blocks an SM).
  *   "chunk"* [1024]     adjacency entries per work item (32..2^20).
@@ -337,7 +339,8 @@ int abcore_get_stats(abcore_ctx *ctx, abcore_stats *out);
  *                       (16, for single peels of large bounds and long rows 1).
  * Batch:
  *   "batch_wave"* [-1]  chains per wave (0..32; 0: all at once); -1: 4, 8 or 16 by the graph's size, and
- *                       read as that number.
+ *                       read as that number. A chain keeps counts, prefixes and a queue of its own,
+ *                       about 16 bytes a vertex; fewer run at once where memory does not hold them.
  *   "batch_plain_below"* [0] pairs with alpha below this run as single peels, not chains.
  *   "batch_seed"* [0]   1: seed each chain from the finished chain of the next smaller alpha.
  *   "packed_counts" [1] chains keep 16-bit counts whenever every degree fits.
