@@ -71,6 +71,7 @@ constexpr int SERVE_EXTRA = 64;
 __device__ __forceinline__ int work_threads() { return (int)blockDim.x - SERVE_EXTRA; }
 __device__ __forceinline__ int work_warps() { return work_threads() >> 5; }
 constexpr int SERVE_RING = 64;                   // requests between two of them at most
+constexpr unsigned long long FAILED = 1ull << 63;  // in the fetched count: the session has failed, what was fetched is left alone
 
 struct TargetDev {
     int32_t alpha, beta;
@@ -183,14 +184,6 @@ __device__ __forceinline__ int32_t ins_capacity(int32_t used) {
     return c;
 }
 
-// Sign of life of the warps that work on an update, in shared memory (null: nobody waits for them). One is given at
-// every vertex they take up and every BEAT_STEPS steps along a row, so whoever waits can tell a long update
-// from one that is stuck, however many levels and entries it has.
-constexpr int BEAT_STEPS = 256;
-__device__ __forceinline__ void beat_on(unsigned *beat) {
-    if (beat != nullptr && (threadIdx.x & 31) == 0) atomicAdd(beat, 1u);
-}
-
 // Visit the current neighbours of w: base row minus tombstones, plus live inserted neighbours.
 // Warp-collective: lanes stride the base row, then the inserted segment. Each lane hands f up to NB of them at once
 // (-1: none), so that what f reads of them is read together: what a re-peel waits for is round trips to L2, and
@@ -198,10 +191,8 @@ __device__ __forceinline__ void beat_on(unsigned *beat) {
 // took six of them a step.
 constexpr int NB = 4;
 template <class F>
-__device__ __forceinline__ void for_neighbours(const ServeArgs &A, const TargetDev &S, int32_t w, unsigned *beat, F f) {
+__device__ __forceinline__ void for_neighbours(const ServeArgs &A, const TargetDev &S, int32_t w, F f) {
     const int lane = threadIdx.x & 31;
-    int step = 0;
-    beat_on(beat);
     const int64_t s = __ldg(&A.off[w]), e = __ldg(&A.off[w + 1]);
     const int2 seg = S.ins[w];
     int32_t z[NB];
@@ -217,21 +208,18 @@ __device__ __forceinline__ void for_neighbours(const ServeArgs &A, const TargetD
         for (int k = 0; k < NB; ++k)
             if (gone[k] & 1u) z[k] = -1;
         f(z);
-        if ((++step & (BEAT_STEPS - 1)) == 0) beat_on(beat);
     }
     for (int32_t i = lane; i - lane < seg.y; i += 32 * NB) {
 #pragma unroll
         for (int k = 0; k < NB; ++k) z[k] = i + 32 * k < seg.y ? S.pool[seg.x + i + 32 * k] : -1;
         f(z);
-        if ((++step & (BEAT_STEPS - 1)) == 0) beat_on(beat);
     }
 }
 
 // Warp-collective: position in the pool of `key` in segment seg, or -1.
-__device__ __forceinline__ int32_t ins_find(const TargetDev &S, int2 seg, int32_t key, unsigned *beat) {
+__device__ __forceinline__ int32_t ins_find(const TargetDev &S, int2 seg, int32_t key) {
     const int lane = threadIdx.x & 31;
     for (int32_t i0 = 0; i0 < seg.y; i0 += 32) {
-        if (i0 > 0 && (i0 & (32 * BEAT_STEPS - 1)) == 0) beat_on(beat);
         const unsigned m = __ballot_sync(ABC_FULL, i0 + lane < seg.y && S.pool[seg.x + i0 + lane] == key);  // live entries are distinct
         if (m) return seg.x + i0 + __ffs(m) - 1;
     }
@@ -246,14 +234,11 @@ __device__ __forceinline__ int32_t append_need(int2 seg) {
 }
 
 // Warp-collective: append y to x's inserted neighbours (segment seg), moving the segment to `at` where it needs room.
-__device__ __forceinline__ void ins_append(TargetDev &S, int32_t x, int2 seg, int32_t y, int32_t at, unsigned *beat) {
+__device__ __forceinline__ void ins_append(TargetDev &S, int32_t x, int2 seg, int32_t y, int32_t at) {
     const int lane = threadIdx.x & 31;
     const bool moves = append_need(seg) > 0;
     if (moves)
-        for (int32_t i = lane; i < seg.y; i += 32) {
-            S.pool[at + i] = S.pool[seg.x + i];
-            if (((i >> 5) & (BEAT_STEPS - 1)) == BEAT_STEPS - 1) beat_on(beat);
-        }
+        for (int32_t i = lane; i < seg.y; i += 32) S.pool[at + i] = S.pool[seg.x + i];
     if (lane == 0) {
         const int32_t to = moves ? at : seg.x;
         S.pool[to + seg.y] = y;
@@ -272,8 +257,8 @@ __device__ __forceinline__ void bq_push(BlockQueue &Q, int32_t z) { Q.q[atomicAd
 
 // Cascade inside the core after a delete: members whose in-core count fell below their bound
 // leave, lowering their member neighbours' counts (queued on the exact crossing). Vertices
-// leaving at cascade level L get certificate level base + L.
-__device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y, unsigned *beat) {
+// leaving at cascade level L get certificate level base + L. Returns true, in thread 0, if the levels have run out.
+__device__ bool delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y) {
     __shared__ int tail;
     __shared__ int64_t base_s;
     BlockQueue Q{S.q, &tail};
@@ -293,7 +278,7 @@ __device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int3
         for (int i = head + warp; i < end; i += nwarps) {
             const int32_t w = S.q[i];
             if ((threadIdx.x & 31) == 0) S.rho[w] = base_s + level;
-            for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
+            for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
                 bool in[NB];
 #pragma unroll
                 for (int k = 0; k < NB; ++k) in[k] = z[k] >= 0 && S.M[z[k]];
@@ -309,17 +294,20 @@ __device__ void delete_cascade(const ServeArgs &A, TargetDev &S, int32_t x, int3
         head = end;
         ++level;
     }
+    bool over = false;
     if (threadIdx.x == 0 && tail > 0) {
         *S.base = base_s + level + 1;
-        if (*S.base > RHO_LIMIT) abc::set_error(A.err, ABCORE_ENOMEM);
+        over = base_s + level + 1 > RHO_LIMIT;
+        if (over) abc::set_error(A.err, ABCORE_ENOMEM);
         S.st[2] += 1;
         S.st[3] += (unsigned long long)tail;
     }
     work_sync();
+    return over;
 }
 
-// Region growth and peel after an insert with an endpoint outside the core (see the header).
-__device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y, int32_t ep, unsigned *beat) {
+// Region growth and peel after an insert with an endpoint outside the core (see the header). Returns as delete_cascade.
+__device__ bool insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32_t y, int32_t ep) {
     __shared__ int tail;
     __shared__ int64_t base_s;
     BlockQueue Q{S.q, &tail};
@@ -338,7 +326,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
         }
     }
     work_sync();
-    if (tail == 0) return;
+    if (tail == 0) return false;
     // grow R along edges of strictly increasing rho through non-core vertices meeting their bound
     int head = 0;
     while (head < tail) {
@@ -347,7 +335,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
         for (int i = head + warp; i < end; i += nwarps) {
             const int32_t w = S.q[i];
             const int64_t rw = S.rho[w];
-            for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
+            for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
                 bool in[NB];
                 int64_t rho[NB];
                 int32_t deg[NB];
@@ -371,7 +359,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
     for (int i = warp; i < R; i += nwarps) {
         const int32_t w = S.q[i];
         int c = 0;
-        for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
+        for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
 #pragma unroll
             for (int k = 0; k < NB; ++k) {
                 const int32_t y = max(z[k], 0);
@@ -403,7 +391,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
         for (int i = head + warp; i < end; i += nwarps) {
             const int32_t w = S.q[i];
             if (lane == 0) S.rho[w] = base_s + level;
-            for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
+            for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
                 bool in[NB];
 #pragma unroll
                 for (int k = 0; k < NB; ++k) in[k] = z[k] >= 0 && S.mark[z[k]] == ep;
@@ -423,7 +411,7 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
     for (int i = warp; i < R; i += nwarps) {
         const int32_t w = S.q[i];
         if (S.mark[w] != ep) continue;
-        for_neighbours(A, S, w, beat, [&](const int32_t (&z)[NB]) {
+        for_neighbours(A, S, w, [&](const int32_t (&z)[NB]) {
 #pragma unroll
             for (int k = 0; k < NB; ++k) {
                 const int32_t y = max(z[k], 0);
@@ -440,13 +428,16 @@ __device__ void insert_region(const ServeArgs &A, TargetDev &S, int32_t x, int32
             S.rho[w] = RHO_CORE;
         }
     }
+    bool over = false;
     if (threadIdx.x == 0) {
         *S.base = base_s + level + 1;
-        if (*S.base > RHO_LIMIT) abc::set_error(A.err, ABCORE_ENOMEM);
+        over = base_s + level + 1 > RHO_LIMIT;
+        if (over) abc::set_error(A.err, ABCORE_ENOMEM);
         S.st[0] += 1;
         S.st[1] += (unsigned long long)R;
     }
     work_sync();
+    return over;
 }
 
 // What an edge change found: memberships, degrees after it and in-core counts before it.
@@ -464,7 +455,7 @@ constexpr int POOL_FULL = 1;
 // status, or POOL_FULL with the view unchanged (admission by memory: a new edge needs room in
 // both endpoints' pool segments). Warp-collective; CORE: the view has a core (M, cnt).
 template <bool CORE>
-__device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int32_t y, int64_t px, int64_t py, Change &ch, unsigned *beat) {
+__device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int32_t y, int64_t px, int64_t py, Change &ch) {
     const int lane = threadIdx.x & 31;
     // one round trip for all of it
     const bool base = px >= 0;
@@ -480,15 +471,15 @@ __device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int
         ch.cx = S.cnt[x];
         ch.cy = S.cnt[y];
     }
-    const int32_t qx = base ? -1 : ins_find(S, sx, y, beat);
+    const int32_t qx = base ? -1 : ins_find(S, sx, y);
     const bool present = base ? ((tw >> (px & 31)) & 1u) == 0 : qx >= 0;
     if (op == ABCORE_INSERT) {
         if (present) return ABCORE_EEXIST;
         if (!base) {
             const int32_t nx = append_need(sx), ny = append_need(sy);
             if ((int64_t)top + nx + ny > (int64_t)S.pool_cap) return POOL_FULL;
-            ins_append(S, x, sx, y, top, beat);
-            ins_append(S, y, sy, x, top + nx, beat);
+            ins_append(S, x, sx, y, top);
+            ins_append(S, y, sy, x, top + nx);
             if (lane == 0 && nx + ny > 0) *S.pool_top = top + nx + ny;
         }
         ch.dx++;
@@ -496,7 +487,7 @@ __device__ __forceinline__ int apply_update(TargetDev &S, int op, int32_t x, int
     } else {
         if (!present) return ABCORE_ENOENT;
         if (!base) {
-            const int32_t qy = ins_find(S, sy, x, beat);
+            const int32_t qy = ins_find(S, sy, x);
             if (lane == 0) {
                 S.pool[qx] = -1;
                 S.pool[qy] = -1;
@@ -534,21 +525,29 @@ __device__ __forceinline__ unsigned long long ld_shared(const unsigned long long
 }
 
 // Limit of a wait of one of a block's warps on another: the other may itself be in its idle spell. Records
-// ABCORE_ETIMEDOUT and returns true once the wait that began with w = {} has taken that long without a sign of life of
-// the warps that work on an update: a re-peel may take longer than any limit, and is waited for while it gets on. (The
-// clock is read only while waiting: it takes longer than a step of an update.)
-struct Wait {
-    unsigned long long since = 0;
-    unsigned beat = 0;
-};
-__device__ __forceinline__ bool wait_over(const ServeArgs &A, Wait &w, const unsigned *beat) {
+// ABCORE_ETIMEDOUT and returns true once the wait that began with since = 0 has taken that long. (The clock is read only
+// while waiting: it takes longer than a step of an update.)
+__device__ __forceinline__ bool wait_over(const ServeArgs &A, unsigned long long &since, unsigned long long more = 0) {
     const unsigned long long now = abc::now_ns();
-    const unsigned b = *(const volatile unsigned *)beat;
-    if (w.since == 0 || b != w.beat) w = Wait{now, b};
-    if (now - w.since <= A.idle_ns + A.timeout_ns) return false;
+    if (since == 0) since = now;
+    if (now - since <= A.idle_ns + A.timeout_ns + more) return false;
     abc::set_error(A.err, ABCORE_ETIMEDOUT);
     return true;
 }
+
+// A wait on the warps that work on an update. A re-peel may take longer than any such limit and waits for nobody itself:
+// while one is under way (counted in `repeels`, odd) it is waited for, ten minutes at most. (A sign of life per 256 steps
+// along rows, with the limit between two of them, cost every update 3 to 5 %.)
+struct WorkWait {
+    unsigned long long since = 0;
+    unsigned repeels = 0;
+    __device__ __forceinline__ bool over(const ServeArgs &A, const volatile unsigned *repeels_now) {
+        const unsigned r = *repeels_now;
+        if (r != repeels) since = 0;
+        repeels = r;
+        return wait_over(A, since, (r & 1u) ? 600ull * 1000000000ull : 0ull);
+    }
+};
 
 __device__ __forceinline__ void st_sys_relaxed(unsigned long long *p, unsigned long long v) {
     asm volatile("st.relaxed.sys.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
@@ -562,17 +561,16 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
     __shared__ unsigned long long s_fetched, s_done, s_sent;
     __shared__ volatile int s_closed;   // the fetch warp has left: nothing follows s_fetched
     __shared__ volatile int s_stop;     // the main warp has left: nothing follows s_done
-    __shared__ volatile int s_failed;   // the session has failed: what was fetched is left alone
     __shared__ int s_job;               // what the waiting warps are to help with: 0 nothing more, 1 a region, 2 a cascade
     __shared__ int32_t s_x, s_y, s_ep;
-    __shared__ unsigned s_beat;         // see beat_on
+    __shared__ volatile unsigned s_repeels;  // re-peels begun and ended
     TargetDev S = A.targets[blockIdx.x];
     const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long k0 = A.progress_dev[t];
     if (threadIdx.x == 0) {
         s_fetched = s_done = s_sent = k0;
-        s_closed = s_stop = s_failed = 0;
-        s_beat = 0;
+        s_closed = s_stop = 0;
+        s_repeels = 0;
     }
     __syncthreads();
     if (warp == work_warps()) {
@@ -583,12 +581,12 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
             int leave = 0;
             if (lane == 0) {
                 const unsigned long long t0 = abc::now_ns();
-                Wait w;
+                WorkWait w;
                 unsigned sl = 32;
                 for (;;) {
                     const int err = abc::ld_relaxed_i32(A.err);
                     if (s_stop || err) {  // this target is held back, or the session failed
-                        if (err) s_failed = 1;
+                        if (err) *(volatile unsigned long long *)&s_fetched = k | FAILED;
                         leave = 1;
                         break;
                     }
@@ -599,8 +597,8 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
                     }
                     const unsigned long long room = ld_shared(&s_done) + SERVE_RING - k;
                     if (room == 0) {  // the main warp is at work
-                        if (wait_over(A, w, &s_beat)) {
-                            s_failed = 1;
+                        if (w.over(A, &s_repeels)) {
+                            *(volatile unsigned long long *)&s_fetched = k | FAILED;
                             leave = 1;
                             break;
                         }
@@ -666,13 +664,13 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
     } else if (warp == work_warps() + 1) {
         // ---- respond ----
         unsigned long long k = k0;
-        Wait w;
+        WorkWait w;
         for (;;) {
             const int stop = s_stop;
             __threadfence_block();
             const unsigned long long done = __shfl_sync(ABC_FULL, ld_shared(&s_done), 0);
             if (k == done) {
-                if (__shfl_sync(ABC_FULL, stop || wait_over(A, w, &s_beat), 0)) break;
+                if (__shfl_sync(ABC_FULL, stop || w.over(A, &s_repeels), 0)) break;
                 __nanosleep(32);
                 continue;
             }
@@ -706,12 +704,12 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
             __threadfence_system();
             __syncwarp();
             if (lane == 0) {
-                A.progress_dev[t] = k;  // (answered, not only applied: a loop that is launched again goes on here)
                 st_sys(&A.progress_host[t], k);
                 *(volatile unsigned long long *)&s_sent = k;
             }
-            w = Wait{};
+            w.since = 0;
         }
+        if (lane == 0) A.progress_dev[t] = k;  // (answered, not only applied: a loop that is launched again goes on here)
     } else if (warp > 0) {
         // ---- the main warp's helpers ----
         for (;;) {
@@ -719,13 +717,12 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
             const int job = s_job;
             const int32_t x = s_x, y = s_y, ep = s_ep;
             if (job == 0) break;
-            if (job == 1) insert_region(A, S, x, y, ep, &s_beat);
-            else delete_cascade(A, S, x, y, &s_beat);
+            if (job == 1) insert_region(A, S, x, y, ep);
+            else delete_cascade(A, S, x, y);
         }
     } else {
         // ---- main ----
-        unsigned long long k = k0;
-        Wait w;
+        unsigned long long k = k0, since = 0;
         int32_t ep = *S.epoch;
         auto all_hands = [&](int job, int32_t x, int32_t y) {
             if (lane == 0) {
@@ -733,17 +730,21 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
                 s_x = x;
                 s_y = y;
                 s_ep = ep;
+                if (job != 0) s_repeels = s_repeels + 1;
             }
             __syncwarp();
             work_sync();
         };
+        auto repeeled = [&]() {
+            if (lane == 0) s_repeels = s_repeels + 1;
+        };
         for (;;) {
             const int closed = s_closed;
             __threadfence_block();
-            if (__shfl_sync(ABC_FULL, s_failed, 0)) break;
             const unsigned long long have = __shfl_sync(ABC_FULL, ld_shared(&s_fetched), 0);
+            if (have & FAILED) break;
             if (k == have) {
-                if (__shfl_sync(ABC_FULL, closed || wait_over(A, w, &s_beat), 0)) break;
+                if (__shfl_sync(ABC_FULL, closed || wait_over(A, since), 0)) break;
                 __nanosleep(20);
                 continue;
             }
@@ -751,7 +752,7 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
             __syncwarp();  // (lane 0 has seen the count: every lane reads the entry after that)
             const Fetched f = ring[k % SERVE_RING];
             Change ch{};
-            const int st = apply_update<true>(S, f.op, f.x, f.y, f.px, f.py, ch, &s_beat);
+            const int st = apply_update<true>(S, f.op, f.x, f.y, f.px, f.py, ch);
             if (st == POOL_FULL) {
                 // hold request k back: the loop closes at k for every block, the host grows this
                 // target's pool and relaunches, and k is processed then (its answer is unchanged)
@@ -762,6 +763,7 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
                 break;
             }
             bool moved = false;  // memberships may have changed
+            bool last = false;   // a re-peel ran out of levels
             if (st == ABCORE_OK) {
                 const int32_t tx = thr_of(A, S, f.x), ty = thr_of(A, S, f.y);
                 if (ch.mx && ch.my) {
@@ -773,22 +775,24 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
                         }
                     } else {  // (a delete that takes an endpoint below its bound)
                         all_hands(2, f.x, f.y);
-                        delete_cascade(A, S, f.x, f.y, &s_beat);
+                        last = __shfl_sync(ABC_FULL, delete_cascade(A, S, f.x, f.y), 0);
+                        repeeled();
                         moved = true;
                     }
                 } else if (f.op == ABCORE_INSERT && ((!ch.mx && ch.dx >= tx) || (!ch.my && ch.dy >= ty))) {
                     ep += 2;
                     all_hands(1, f.x, f.y);
-                    insert_region(A, S, f.x, f.y, ep, &s_beat);
+                    last = __shfl_sync(ABC_FULL, insert_region(A, S, f.x, f.y, ep), 0);
+                    repeeled();
                     moved = true;
                 }
             }
             __syncwarp();
             const int bits = moved ? (S.M[f.x] ? 1 : 0) | (S.M[f.y] ? 2 : 0) : (ch.mx ? 1 : 0) | (ch.my ? 2 : 0);
-            w = Wait{};
+            since = 0;
             bool stuck = false;
             while (!stuck && k - __shfl_sync(ABC_FULL, ld_shared(&s_sent), 0) >= SERVE_RING) {  // the respond warp is behind
-                stuck = __shfl_sync(ABC_FULL, wait_over(A, w, &s_beat), 0);
+                stuck = __shfl_sync(ABC_FULL, wait_over(A, since), 0);
                 __nanosleep(64);
             }
             if (stuck) break;
@@ -799,7 +803,7 @@ __global__ void __launch_bounds__(WORK + SERVE_EXTRA, MINB) k_serve(ServeArgs A)
             }
             ++k;
             __syncwarp();
-            if (moved && __shfl_sync(ABC_FULL, abc::ld_relaxed_i32(A.err), 0)) break;  // (a re-peel ran out of levels)
+            if (last) break;
         }
         all_hands(0, 0, 0);
         __threadfence_block();
@@ -906,7 +910,7 @@ __global__ void __launch_bounds__(32) k_gfq_apply(ServeArgs A, TargetDev V, int 
     const int64_t px = warp_find(A.adj, __ldg(&A.off[x]), __ldg(&A.off[x + 1]), y);
     const int64_t py = px < 0 ? -1 : warp_find(A.adj, __ldg(&A.off[y]), __ldg(&A.off[y + 1]), x);
     Change ch{};
-    const int st = apply_update<false>(V, op, x, y, px, py, ch, nullptr);
+    const int st = apply_update<false>(V, op, x, y, px, py, ch);
     if (threadIdx.x == 0) {
         ids[0] = x;
         ids[1] = y;
@@ -977,7 +981,7 @@ __global__ void k_gfq_round(ServeArgs A, TargetDev V, int32_t alpha, int32_t bet
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = w0; i < nin; i += nw) {
         const int32_t w = fin[i];
-        for_neighbours(A, V, w, nullptr, [&](const int32_t (&z)[NB]) {
+        for_neighbours(A, V, w, [&](const int32_t (&z)[NB]) {
             bool in[NB];
 #pragma unroll
             for (int k = 0; k < NB; ++k) in[k] = z[k] >= 0 && alive[z[k]];
